@@ -264,8 +264,9 @@ nb_status nb_jacobi_diagonal(nb_ctx *ctx, double *minv_dev);
 nb_status nb_solve_stats(const nb_ctx *ctx, int *iters, int *outer);
 
 /* Select the ax_e kernel: 0 = automatic (fastest FP64-accurate kernel),
- * 1 = native FP64 layer kernel, 2 = double-float (FP32-pair) kernel.  All
- * variants meet the same accuracy contract. */
+ * 1 = native FP64 layer kernel, 2 = the kernel on the integer and FP32 pipes
+ * (fixed-point pairs; the automatic choice at every n).  All variants meet
+ * the same accuracy contract. */
 nb_status nb_set_ax_variant(nb_ctx *ctx, int variant);
 
 /* --------------------------------------------------------------------- */

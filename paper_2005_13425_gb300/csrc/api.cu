@@ -127,7 +127,7 @@ static const char *const slab_refusal =
 void free_ctx(nb_ctx *c) {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    void *ptrs[] = {c->d_D, c->d_gxyz, c->d_mask, c->d_Df, c->d_gxyz_df, c->d_gxyz32, c->d_minv,
+    void *ptrs[] = {c->d_D, c->d_gxyz, c->d_mask, c->d_Df, c->d_gxyz_fx, c->d_gxyz32, c->d_minv,
                     c->d_r, c->d_p, c->d_w, c->d_x, c->d_partials, c->d_sc, c->d_hist,
                     c->d_r32, c->d_p32, c->d_w32, c->d_z32};
     for (void *p : ptrs)
@@ -229,7 +229,7 @@ nb_status nb_setup(nb_ctx **out, nb_box mesh, int n, const double *D, const doub
         if ((e = cudaMemcpyAsync(c->d_mask, mask, c->m.npts, cudaMemcpyHostToDevice, c->stream)) != cudaSuccess)
             return bail(cuda_fail(e, "copy mask"));
     }
-    if ((s = prepare_df(c)) != NB_OK) return bail(s);
+    if ((s = prepare_fx(c)) != NB_OK) return bail(s);
     if (prec == NB_MIXED && (s = prepare_fp32(c)) != NB_OK) return bail(s);
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(cuda_fail(e, "setup sync"));
     *out = c;
@@ -278,7 +278,7 @@ nb_status nb_setup_box(nb_ctx **out, nb_box mesh, int n, double amp, const doubl
     cudaFree(d_bad);
     if (s != NB_OK) return bail(s);
     if (bad) return bail(fail(NB_ERR_ARG, "the perturbed map folds: |J| <= 0 somewhere"));
-    if ((s = prepare_df(c)) != NB_OK) return bail(s);
+    if ((s = prepare_fx(c)) != NB_OK) return bail(s);
     if (prec == NB_MIXED && (s = prepare_fp32(c)) != NB_OK) return bail(s);
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(cuda_fail(e, "setup sync"));
     *out = c;

@@ -1,8 +1,7 @@
-// Core of the double-float ax_e (Listing 1, arXiv 2005.13425 Sec. III) shared
-// by the single-problem kernel (ax_df.cu) and the batched engine
-// (engine.cu): derivative-matrix constants, the line products (plain and
-// even-odd) and the per-element operator df_element().  See ax_df.cu for
-// the arithmetic and thread layout.
+// Double-float ax_e (Listing 1, arXiv 2005.13425 Sec. III) on FP32 pairs
+// (df.cuh) for the batched engine (engine.cu), the CG head on boxes of few
+// elements (ax_df.cu) and the measurement probe (probe_tc.cu): derivative-matrix constants, the even-odd line product and
+// one element of the operator.
 #pragma once
 
 #include "df.cuh"
@@ -10,12 +9,6 @@
 #include "reduce.cuh"
 
 namespace nekgb {
-
-template <int N>
-struct DfMat {
-    float h[N * N];   // h[m*N + l] + l_[m*N + l] = D(m, l)
-    float l[N * N];
-};
 
 // Even-odd form of a centro-antisymmetric matrix M (M(N-1-m, N-1-l) =
 // -M(m,l), which holds for the GLL derivative matrix and its transpose).
@@ -85,32 +78,8 @@ __device__ __forceinline__ int line_of(int task, int &stride) {
     return a0 + N * a1;
 }
 
-// out(base + m*stride) = sum_l M(m,l) in(base + l*stride), M = D or D^T,
-// n compensated dot products of n terms.
-template <int N, bool TR>
-__device__ __forceinline__ void line_plain(const float2 *in, float2 *out, int base, int stride,
-                                           const DfMat<N> &D) {
-    float xh[N], xl[N];
-#pragma unroll
-    for (int l = 0; l < N; l++) {
-        const float2 v = in[base + l * stride];
-        xh[l] = v.x;
-        xl[l] = v.y;
-    }
-#pragma unroll
-    for (int m = 0; m < N; m++) {
-        const int i0 = TR ? m : m * N;
-        dfa::Acc acc = dfa::first(D.h[i0], D.l[i0], xh[0], xl[0]);
-#pragma unroll
-        for (int l = 1; l < N; l++) {
-            const int il = TR ? l * N + m : m * N + l;
-            dfa::fma(acc, D.h[il], D.l[il], xh[l], xl[l]);
-        }
-        out[base + m * stride] = dfa::norm(acc);
-    }
-}
-
-// The same line product in even-odd form (see EoMat): pair sums and
+// out(base + m*stride) = sum_l M(m,l) in(base + l*stride) in even-odd form
+// (see EoMat): pair sums and
 // differences, then 2 dot products of N/2 terms per output pair.
 template <int N>
 __device__ __forceinline__ void line_eo(const float2 *in, float2 *out, int base, int stride,
@@ -152,57 +121,19 @@ __device__ __forceinline__ void line_eo(const float2 *in, float2 *out, int base,
     }
 }
 
-template <int N, bool EO>
-struct DfConsts;
-template <int N>
-struct DfConsts<N, false> { using type = DfMat<N>; };
-template <int N>
-struct DfConsts<N, true> { using type = DfEo<N>; };
-
-
-// Per-element arguments of df_element (pointers already offset to the element).
-struct DfElemIO {
-    const double *u;    // MODE 0: input
-    const double *r;    // MODE 1: residual
-    double *p;          // MODE 1: search direction (updated in place)
-    double *x;          // MODE 1: iterate (owed update applied when xa != 0)
-    const double *minv; // MODE 1: Jacobi inverse diagonal (z = minv r), or null
-    double *w;          // output
-    const float2 *g;    // gxyz pairs [6][n^3] of the element, scaled by 2^-(gexp-1023)
-};
-
 // Points of an element per thread of a T-thread CTA in the pointwise phases.
 template <int N, int T>
 __host__ __device__ constexpr int df_points_per_thread() {
     return (N * N * N + T - 1) / T;
 }
 
-// This thread's point-face masks (point_faces of q = threadIdx.x + k T),
-// computed once per kernel for df_element's fused CG head.
+// w = ax_e(u) on one element in double-float arithmetic, executed by the whole
+// CTA (every thread must call it; it contains barriers).  u, w: the element's
+// points, g: its gxyz pairs [6][n^3], unscaled.  sm holds 6 n^3 pairs, s_emax
+// is a shared int that must be 0 on entry (left 0 on exit).
 template <int N, int T>
-__device__ __forceinline__ void df_point_masks(unsigned *pf) {
-#pragma unroll
-    for (int k = 0; k < df_points_per_thread<N, T>(); k++) {
-        const int q = threadIdx.x + k * T;
-        pf[k] = q < N * N * N ? point_faces<N>(q) : 0u;
-    }
-}
-
-// One element of ax_e in double-float arithmetic, executed by the whole CTA
-// (every thread must call it; it contains barriers).  sm holds 6 n^3 pairs,
-// s_emax is a shared int that must be 0 on entry (left 0 on exit).
-// MODE 1 is the CG head: x += xa p, p = r + beta p, w = ax_e(p); with fuse,
-// box-face points of w are zeroed and the element's share of <w,p>_c (the
-// local products, see the final loop) is added to dot; pf holds the thread's point-face masks (df_point_masks; null:
-// computed per point) and (ex, ey, ez) is the element's position in the box m.  The geometric
-// factors and x are loaded with the streaming (evict-first) cache policy:
-// they are not read again in the iteration, which keeps w and p in L2 for
-// the dssum and update kernels that follow.
-template <int N, int MODE, bool EO, int T = ax_df_threads(N)>
-__device__ __forceinline__ void df_element(const DfElemIO &io, double beta, double xa, bool fuse,
-                                           int gexp, const Mesh &m, int ex, int ey, int ez,
-                                           const typename DfConsts<N, EO>::type &D, float2 *sm,
-                                           int *s_emax, double &dot, const unsigned *pf = nullptr) {
+__device__ __forceinline__ void df_element(const double *u, double *w, const float2 *g, const DfEo<N> &D, float2 *sm,
+                                           int *s_emax) {
     constexpr int N2 = N * N, N3 = N * N * N;
     float2 *U = sm;            // input pairs; later the r-partial of w
     float2 *W0 = sm + N3;      // wr -> ur
@@ -214,38 +145,11 @@ __device__ __forceinline__ void df_element(const DfElemIO &io, double beta, doub
     const int t = threadIdx.x;
     // ---- stage the element (raw FP64 first, to find its scale)
     int emax = 0;
-    // x += alpha p of the previous iteration, then p = z + beta p; the
-    // preconditioner and owed-update branches are uniform, so they are taken
-    // outside the point loops
-    auto stage = [&](double v, int q) {
+    for (int q = t; q < N3; q += T) {
+        const double v = __ldg(u + q);
         raw[q] = v;
         const int exb = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
         emax = exb > emax ? exb : emax;
-    };
-    if (MODE == 0) {
-        for (int q = t; q < N3; q += T) stage(__ldg(io.u + q), q);
-    } else if (io.minv) {
-        for (int q = t; q < N3; q += T) {
-            const double pold = io.p[q];
-            if (xa != 0.0) __stcs(io.x + q, fma(xa, pold, __ldcs(io.x + q)));
-            const double v = fma(beta, pold, io.r[q] * io.minv[q]);
-            io.p[q] = v;
-            stage(v, q);
-        }
-    } else if (xa != 0.0) {
-        for (int q = t; q < N3; q += T) {
-            const double pold = io.p[q];
-            __stcs(io.x + q, fma(xa, pold, __ldcs(io.x + q)));
-            const double v = fma(beta, pold, io.r[q]);
-            io.p[q] = v;
-            stage(v, q);
-        }
-    } else {
-        for (int q = t; q < N3; q += T) {
-            const double v = fma(beta, io.p[q], io.r[q]);
-            io.p[q] = v;
-            stage(v, q);
-        }
     }
     emax = __reduce_max_sync(0xffffffffu, emax);
     if ((t & 31) == 0) atomicMax(s_emax, emax);
@@ -253,9 +157,8 @@ __device__ __forceinline__ void df_element(const DfElemIO &io, double beta, doub
     int eu = *s_emax;
     eu = eu < 1 ? 1 : (eu > 2046 ? 2046 : eu);
     // u is scaled by 2^(1023-eu) so the element's max is in [1,2); w is
-    // scaled back by 2^(eu-1023) and by the gxyz scale 2^(gexp-1023)
-    const int sh_in = 1023 - eu;
-    const int sh_out = (eu - 1023) + (gexp - 1023);
+    // scaled back by 2^(eu-1023)
+    const int sh_in = 1023 - eu, sh_out = eu - 1023;
     for (int q = t; q < N3; q += T) U[q] = dfa::split_scaled(raw[q], sh_in);  // own entries only
     __syncthreads();
 
@@ -263,16 +166,11 @@ __device__ __forceinline__ void df_element(const DfElemIO &io, double beta, doub
     for (int task = t; task < 3 * N2; task += T) {
         int stride;
         const int base = line_of<N>(task, stride);
-        float2 *Wd = task < N2 ? W0 : (task < 2 * N2 ? W1 : W2);
-        if constexpr (EO)
-            line_eo<N>(U, Wd, base, stride, D.fwd);
-        else
-            line_plain<N, false>(U, Wd, base, stride, D);
+        line_eo<N>(U, task < N2 ? W0 : (task < 2 * N2 ? W1 : W2), base, stride, D.fwd);
     }
     __syncthreads();
 
     // ---- geometric contraction, pointwise, in place
-    const float2 *g = io.g;
     for (int q = t; q < N3; q += T) {
         const float2 wr = W0[q], ws = W1[q], wt = W2[q];
         const float2 g0 = __ldcs(g + q), g1 = __ldcs(g + N3 + q), g2 = __ldcs(g + 2 * N3 + q);
@@ -296,41 +194,14 @@ __device__ __forceinline__ void df_element(const DfElemIO &io, double beta, doub
     for (int task = t; task < 3 * N2; task += T) {
         int stride;
         const int base = line_of<N>(task, stride);
-        const float2 *Ud = task < N2 ? W0 : (task < 2 * N2 ? W1 : W2);
-        float2 *Pd = task < N2 ? U : (task < 2 * N2 ? P1 : P2);
-        if constexpr (EO)
-            line_eo<N>(Ud, Pd, base, stride, D.bwd);
-        else
-            line_plain<N, true>(Ud, Pd, base, stride, D);
+        line_eo<N>(task < N2 ? W0 : (task < 2 * N2 ? W1 : W2), task < N2 ? U : (task < 2 * N2 ? P1 : P2), base,
+                   stride, D.bwd);
     }
     __syncthreads();
 
     // ---- w = r-partial + s-partial + t-partial, scaled back, FP64 out
-    if (MODE == 1 && fuse) {
-        // Dirichlet points are zeroed before dssum (their sum is then +0, as
-        // mask-after-dssum gives).  <w,p>_c is summed here over all local
-        // points: p is continuous, so sum_g (sum_copies w) p_g equals the
-        // sum of the local products before assembly.
-        const unsigned bf = box_faces(ex, ey, ez, m);
-#pragma unroll
-        for (int k = 0; k < df_points_per_thread<N, T>(); k++) {
-            const int q = t + k * T;
-            if (df_points_per_thread<N, T>() * T != N3 && q >= N3) break;
-            const float2 s = dfa::add(dfa::add(U[q], P1[q]), P2[q]);
-            double wv = dfa::join_scaled(s, sh_out);
-            const unsigned f = pf ? pf[k] : point_faces<N>(q);
-            if (f & bf)
-                wv = 0.0;
-            else
-                dot = fma(wv, io.p[q], dot);
-            io.w[q] = wv;
-        }
-    } else {
-        for (int q = t; q < N3; q += T) {
-            const float2 s = dfa::add(dfa::add(U[q], P1[q]), P2[q]);
-            io.w[q] = dfa::join_scaled(s, sh_out);
-        }
-    }
+    for (int q = t; q < N3; q += T)
+        w[q] = dfa::join_scaled(dfa::add(dfa::add(U[q], P1[q]), P2[q]), sh_out);
     if (t == 0) *s_emax = 0;
     __syncthreads();
 }
@@ -352,21 +223,6 @@ inline void eo_consts(const double *Dm, bool tr, EoMat<N> &E) {
         }
     }
     for (int l = 0; l <= H; l++) put((N & 1) ? M(H, l) : 0.0, E.ch[l], E.cl[l]);
-}
-
-// Fill the kernel-parameter constants for D (plain pairs or even-odd form).
-template <int N, bool EO>
-inline void df_consts(const double *Dh, typename DfConsts<N, EO>::type &D) {
-    if constexpr (EO) {
-        eo_consts<N>(Dh, false, D.fwd);
-        eo_consts<N>(Dh, true, D.bwd);
-    } else {
-        for (int q = 0; q < N * N; q++) {
-            const float h = (float)Dh[q];
-            D.h[q] = h;
-            D.l[q] = (float)(Dh[q] - (double)h);
-        }
-    }
 }
 
 }  // namespace nekgb

@@ -30,8 +30,7 @@
 namespace nekgb {
 
 nb_status launch_ax_fp64(nb_ctx *c, const double *u, double *w, int mode);
-nb_status launch_ax_df(nb_ctx *c, const double *u, double *w, int mode);
-bool df_supported(int n);
+nb_status launch_ax_fx(nb_ctx *c, const double *u, double *w, int mode);
 nb_status launch_dssum_sc(nb_ctx *c, double *w, const CgScalars *sc);
 nb_status launch_dssum_cg(nb_ctx *c);
 nb_status launch_mask_sc(nb_ctx *c, double *w, const CgScalars *sc);
@@ -279,16 +278,17 @@ static nb_status launch_update(nb_ctx *c) {
     return NB_OK;
 }
 
-static bool use_df(const nb_ctx *c) {
-    return (c->ax_variant == 0 || c->ax_variant == 2) && c->d_gxyz_df && df_supported(c->m.n);
+static bool use_fx(const nb_ctx *c) {
+    return (c->ax_variant == 0 || c->ax_variant == 2) && c->d_gxyz_fx;
 }
 
 nb_status launch_ax(nb_ctx *c, const double *u, double *w) {
-    return use_df(c) ? launch_ax_df(c, u, w, 0) : launch_ax_fp64(c, u, w, 0);
+    return use_fx(c) ? launch_ax_fx(c, u, w, 0) : launch_ax_fp64(c, u, w, 0);
 }
 
 nb_status launch_ax_cg(nb_ctx *c) {
-    return use_df(c) ? launch_ax_df(c, nullptr, nullptr, 1) : launch_ax_fp64(c, nullptr, nullptr, 1);
+    if (use_fx(c) && c->two_kernel && c->d_gxyz_df) return launch_df_head(c);
+    return use_fx(c) ? launch_ax_fx(c, nullptr, nullptr, 1) : launch_ax_fp64(c, nullptr, nullptr, 1);
 }
 
 nb_status ensure_cg_workspace(nb_ctx *c) {
@@ -394,7 +394,7 @@ nb_status cg_solve_fp64(nb_ctx *c, const double *f, double *x, double tol, int m
     if ((s = ensure_cg_workspace(c)) != NB_OK) return s;
     if ((s = ensure_hist(c, maxit)) != NB_OK) return s;
     c->fused_cg = c->d_mask == nullptr;
-    c->two_kernel = c->fused_cg && !c->d_minv && use_df(c);
+    c->two_kernel = c->fused_cg && !c->d_minv && use_fx(c);
     const size_t bytes = sizeof(double) * c->m.npts;
     CgScalars init{};
     init.tol = tol;

@@ -767,18 +767,9 @@ eng_m_outer_ax(ProbDesc *__restrict__ desc, const int2 *__restrict__ tiles, cons
         const Mesh m = P.m;
         const int64_t e0 = (int64_t)tile.y * P.te;
         const int64_t e1 = e0 + P.te < m.E ? e0 + P.te : m.E;
-        double dot = 0.0;
         for (int64_t e = e0; e < e1; e++) {
             const int64_t eb = e * N3;
-            DfElemIO io;
-            io.u = P.x + eb;
-            io.r = nullptr;
-            io.p = nullptr;
-            io.x = nullptr;
-            io.minv = nullptr;
-            io.w = P.w + eb;
-            io.g = P.g + e * 6 * N3;
-            df_element<N, 0, true, T>(io, 0.0, 0.0, false, 1023, m, 0, 0, 0, D, sm, &s_emax, dot);
+            df_element<N, T>(P.x + eb, P.w + eb, P.g + e * 6 * N3, D, sm, &s_emax);
         }
     }
 }

@@ -110,23 +110,27 @@ struct nb_ctx {
     nekgb::Mesh m;
     nb_precision prec;
     cudaStream_t stream;
-    int ax_variant;       // 0 auto, 1 fp64, 2 double-float
+    int ax_variant;       // 0 auto, 1 fp64, 2 fixed-point pairs
     double D_host[nekgb::kMaxN * nekgb::kMaxN];
     // operator data
     double *d_D = nullptr;      // n*n, D[i*n+l]
     double *d_gxyz = nullptr;   // [E][6][n^3]
     uint8_t *d_mask = nullptr;  // [E][n^3] or null (box mask)
     float *d_Df = nullptr;      // D as double-float pairs / fp32 (2*n*n)
-    float2 *d_gxyz_df = nullptr;  // [E][6][n^3] (hi,lo) pairs for double-float ax
+    int4 *d_gxyz_fx = nullptr;  // [E][3][n^3] fixed-point pairs of gxyz, two per entry (ax_fx_core.cuh)
+    int *d_ge = nullptr;        // [E] their exponents (in d_gxyz_fx's allocation)
+    std::vector<int4> fx_tab;   // D's tables for that kernel (FxEo<n> or FxMat<n>)
+    int fx_dot_shift0 = 0, fx_dot_lim = 0;   // scale of the head's exact <w,p>_c (ax_fx.cu)
     float *d_gxyz32 = nullptr;  // [E][6][n^3] fp32 for the mixed inner solve
-    int gxyz_exp = 1023;
+    float2 *d_gxyz_df = nullptr;  // [E][6][n^3] float pairs for the CG head on few elements (ax_df.cu; in d_gxyz_fx's allocation), or null
+    int gxyz_exp = 1023;        // biased exponent of max|gxyz|
     bool d_eo = false;          // D is centro-antisymmetric: even-odd line products
     bool is_box = false;        // built by nb_setup_box (coordinates known)
     // slab of a z-partitioned box (nb_setup_slab): element layers
     // slab_z0 .. slab_z0 + m.ez - 1 of a box slab_ez_global layers high
     bool slab = false;
     int slab_z0 = 0, slab_ez_global = 0;
-    double box_amp = 0.0, box_s[3] = {0, 0, 0};        // biased exponent of max|gxyz| (pairs are scaled by 2^-(gxyz_exp-1023))
+    double box_amp = 0.0, box_s[3] = {0, 0, 0};
     // CG workspace
     double *d_r = nullptr, *d_p = nullptr, *d_w = nullptr, *d_x = nullptr;
     double *d_partials = nullptr;
@@ -183,7 +187,7 @@ struct LaunchTimer {
 nb_status harvest_timing(nb_ctx *c);
 
 // ---------------------------------------------------------------- kernels
-// ax_e (ax_fp64.cu / ax_df.cu)
+// ax_e (ax_fp64.cu / ax_fx.cu)
 nb_status launch_ax(nb_ctx *c, const double *u, double *w);
 // CG fused: p = r + beta p, w = ax_e(p)   (beta from CgScalars)
 nb_status launch_ax_cg(nb_ctx *c);
@@ -212,7 +216,10 @@ nb_status cg_solve_mixed(nb_ctx *c, const double *f, double *x, double tol, int 
                          int *iters, double *relres);
 nb_status ensure_cg_workspace(nb_ctx *c);
 nb_status set_preconditioner(nb_ctx *c, int kind);   // precond.cu
-nb_status prepare_df(nb_ctx *c);   // double-float copies of D and gxyz
+nb_status prepare_fx(nb_ctx *c);   // fixed-point pairs of gxyz
+bool df_head_elements(int64_t E, int n);
+nb_status prepare_df(nb_ctx *c);   // float pairs of gxyz (few elements)
+nb_status launch_df_head(nb_ctx *c);
 bool centro_antisymmetric(const double *D, int n);
 nb_status prepare_fp32(nb_ctx *c); // fp32 copy of gxyz for the mixed solve
 

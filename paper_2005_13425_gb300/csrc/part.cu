@@ -38,7 +38,7 @@ namespace nekgb {
 nb_status host_gll(int n, double *xi, double *w);
 nb_status host_dmat(int n, const double *x, double *D);
 nb_status launch_box_geometry(nb_ctx *c, double amp, const double *s, int *bad_dev);
-nb_status prepare_df(nb_ctx *c);
+nb_status prepare_fx(nb_ctx *c);
 nb_status check_mesh(nb_box mesh, int n);
 nb_status new_ctx(nb_ctx **out, nb_box mesh, int n, nb_precision prec, void *stream);
 void free_ctx(nb_ctx *c);
@@ -256,7 +256,7 @@ nb_status nb_setup_slab(nb_ctx **out, nb_box global, int z0, int z1, int n, doub
     cudaFree(d_bad);
     if (s != NB_OK) return bail(s);
     if (bad) return bail(fail(NB_ERR_ARG, "the perturbed map folds: |J| <= 0 somewhere"));
-    if ((s = prepare_df(c)) != NB_OK) return bail(s);
+    if ((s = prepare_fx(c)) != NB_OK) return bail(s);
     if ((s = ensure_cg_workspace(c)) != NB_OK) return bail(s);
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(cuda_fail(e, "setup sync"));
     *out = c;

@@ -115,7 +115,7 @@ def measured_peaks(root: str):
 
 # Sources of the double-float CG head kernel; a recorded DRAM traffic figure
 # is valid only for the sources it was measured on.
-CG_HEAD_SOURCES = ("ax_df.cu", "ax_df_core.cuh", "df.cuh", "reduce.cuh")
+CG_HEAD_SOURCES = ("ax_fx_kernel.cuh", "ax_fx_core.cuh", "fx.cuh", "reduce.cuh")
 
 
 _C_COMMENT = re.compile(r"//[^\n]*|/\*.*?\*/", re.S)
