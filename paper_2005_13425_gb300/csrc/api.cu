@@ -337,7 +337,7 @@ nb_status nb_apply(nb_ctx *c, const double *u, double *w) {
     if (c && c->slab) return fail(NB_ERR_STATE, slab_refusal);
     nb_status s = nb_ax(c, u, w);
     if (s != NB_OK) return s;
-    return launch_dssum(c, w, true);
+    return launch_apply_tail(c, w);
     NB_GUARD_END
 }
 

@@ -18,10 +18,41 @@
 
 namespace nekgb {
 
+// One shared node: its copies added from +0.0 in ascending element order, the
+// sum written back to every copy.  (+0.0) + v equals v except for v = -0.0, so
+// the first add is a sign fix-up done with integer operations; the remaining
+// adds are exact-count loops (no predicated-off FP64 adds on GB300's narrow
+// FP64 pipe).
+template <typename T>
+__device__ __forceinline__ void sum_copies(T *w, const int64_t *idx, int c) {
+    if (c == 2) {
+        const T s = plus_zero(w[idx[0]]) + w[idx[1]];
+        w[idx[0]] = s;
+        w[idx[1]] = s;
+    } else if (c == 4) {
+        T a[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) a[k] = w[idx[k]];
+        T s = plus_zero(a[0]);
+#pragma unroll
+        for (int k = 1; k < 4; k++) s = s + a[k];
+#pragma unroll
+        for (int k = 0; k < 4; k++) w[idx[k]] = s;
+    } else {
+        T a[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) a[k] = w[idx[k]];
+        T s = plus_zero(a[0]);
+#pragma unroll
+        for (int k = 1; k < 8; k++) s = s + a[k];
+#pragma unroll
+        for (int k = 0; k < 8; k++) w[idx[k]] = s;
+    }
+}
+
 // Plain dssum (CG = false) or the fused solver step (CG = true), over the
-// shared nodes grouped by category (faces, edges, vertices; DsCat): each
-// node adds its copies from +0.0 in ascending element order and writes the
-// sum back to every copy.  In the solver the ax_e head has already summed
+// shared nodes grouped by category (faces, edges, vertices; DsCat).  In the
+// solver the ax_e head has already summed
 // <w,p>_c as local products (p is continuous, so the assembled product
 // equals the sum of the unassembled ones); the last CTA here reduces those
 // partials, forms alpha = rho/<w,p>_c and flags a breakdown.  N is the
@@ -34,33 +65,7 @@ dssum_kernel(T *__restrict__ w, DsCat dd, CgScalars *sc, double *partials, int s
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
         int64_t idx[8];
         const int c = cat_copies<N>(q, dd, idx);
-        // (+0.0) + v equals v except for v = -0.0, so the first add is a sign
-        // fix-up done with integer operations; the remaining adds are
-        // exact-count loops (no predicated-off FP64 adds on GB300's narrow
-        // FP64 pipe).
-        if (c == 2) {
-            const T s = plus_zero(w[idx[0]]) + w[idx[1]];
-            w[idx[0]] = s;
-            w[idx[1]] = s;
-        } else if (c == 4) {
-            T a[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) a[k] = w[idx[k]];
-            T s = plus_zero(a[0]);
-#pragma unroll
-            for (int k = 1; k < 4; k++) s = s + a[k];
-#pragma unroll
-            for (int k = 0; k < 4; k++) w[idx[k]] = s;
-        } else {
-            T a[8];
-#pragma unroll
-            for (int k = 0; k < 8; k++) a[k] = w[idx[k]];
-            T s = plus_zero(a[0]);
-#pragma unroll
-            for (int k = 1; k < 8; k++) s = s + a[k];
-#pragma unroll
-            for (int k = 0; k < 8; k++) w[idx[k]] = s;
-        }
+        sum_copies(w, idx, c);
     }
     if (CG) {
         double v[1] = {0.0}, tot[1];
@@ -81,39 +86,71 @@ dssum_kernel(T *__restrict__ w, DsCat dd, CgScalars *sc, double *partials, int s
     }
 }
 
-// Box mask: zero every local point on a face of the box (only those points
-// are visited: two faces per direction, n^2 points per face element).
-__global__ void mask_box_kernel(double *__restrict__ w, Mesh m, const CgScalars *__restrict__ sc) {
-    if (sc && sc->done) return;
+// Local points on the faces of the box (two faces per direction, n^2 points
+// per face element; a point on several faces is listed once for each).
+__host__ __device__ inline int64_t box_face_points(const Mesh &m) {
+    return 2 * (int64_t)m.n * m.n * ((int64_t)m.ey * m.ez + (int64_t)m.ex * m.ez + (int64_t)m.ex * m.ey);
+}
+
+__device__ __forceinline__ int64_t box_face_point(int q, const Mesh &m) {
     const int n = m.n, n2 = n * n;
     const int64_t n3 = (int64_t)n * n * n;
     const int fx = m.ey * m.ez * n2, fy = m.ex * m.ez * n2, fz = m.ex * m.ey * n2;
-    const int total = 2 * (fx + fy + fz);
+    int ex, ey, ez, i, j, k, r;
+    if (q < 2 * fx) {
+        const int side = q / fx;
+        r = q - side * fx;
+        const int pt = r % n2, el = r / n2;
+        ey = el % m.ey; ez = el / m.ey; ex = side ? m.ex - 1 : 0;
+        j = pt % n; k = pt / n; i = side ? n - 1 : 0;
+    } else if (q < 2 * (fx + fy)) {
+        const int qq = q - 2 * fx;
+        const int side = qq / fy;
+        r = qq - side * fy;
+        const int pt = r % n2, el = r / n2;
+        ex = el % m.ex; ez = el / m.ex; ey = side ? m.ey - 1 : 0;
+        i = pt % n; k = pt / n; j = side ? n - 1 : 0;
+    } else {
+        const int qq = q - 2 * (fx + fy);
+        const int side = qq / fz;
+        r = qq - side * fz;
+        const int pt = r % n2, el = r / n2;
+        ex = el % m.ex; ey = el / m.ex; ez = side ? m.ez - 1 : 0;
+        i = pt % n; j = pt / n; k = side ? n - 1 : 0;
+    }
+    const int64_t e = ex + (int64_t)m.ex * (ey + (int64_t)m.ey * ez);
+    return e * n3 + i + n * (j + n * k);
+}
+
+// Box mask: zero every local point on a face of the box (only those points
+// are visited).
+__global__ void mask_box_kernel(double *__restrict__ w, Mesh m, const CgScalars *__restrict__ sc) {
+    if (sc && sc->done) return;
+    const int total = (int)box_face_points(m);
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x)
+        w[box_face_point(q, m)] = 0.0;
+}
+
+// dssum and box mask in one launch: the shared nodes inside the box are
+// summed, and every point on a face of the box is zeroed.  Shared nodes on a
+// face are left to the zeroing, so no point is touched by both and the two
+// halves need no order.  Bound by the gathers' latency; the mask's own launch cost
+// more than its work at every size.  nb_apply, one launch against two: 64
+// elements at n = 8 11.5 and 14.4 us, 504 at n = 16 62.8 and 66.6, 4096 at n = 10
+// 100.4 and 104.6, 32768 at n = 12 1357 and 1359.
+template <int N>
+__global__ void __launch_bounds__(256, 5)
+dssum_mask_kernel(double *__restrict__ w, DsCat dd, Mesh m) {
+    const int nodes = dd.o[7], total = nodes + (int)box_face_points(m);
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
-        int ex, ey, ez, i, j, k, r;
-        if (q < 2 * fx) {
-            const int side = q / fx;
-            r = q - side * fx;
-            const int pt = r % n2, el = r / n2;
-            ey = el % m.ey; ez = el / m.ey; ex = side ? m.ex - 1 : 0;
-            j = pt % n; k = pt / n; i = side ? n - 1 : 0;
-        } else if (q < 2 * (fx + fy)) {
-            const int qq = q - 2 * fx;
-            const int side = qq / fy;
-            r = qq - side * fy;
-            const int pt = r % n2, el = r / n2;
-            ex = el % m.ex; ez = el / m.ex; ey = side ? m.ey - 1 : 0;
-            i = pt % n; k = pt / n; j = side ? n - 1 : 0;
-        } else {
-            const int qq = q - 2 * (fx + fy);
-            const int side = qq / fz;
-            r = qq - side * fz;
-            const int pt = r % n2, el = r / n2;
-            ex = el % m.ex; ey = el / m.ex; ez = side ? m.ez - 1 : 0;
-            i = pt % n; j = pt / n; k = side ? n - 1 : 0;
+        if (q >= nodes) {
+            w[box_face_point(q - nodes, m)] = 0.0;
+            continue;
         }
-        const int64_t e = ex + (int64_t)m.ex * (ey + (int64_t)m.ey * ez);
-        w[e * n3 + i + n * (j + n * k)] = 0.0;
+        int64_t idx[8];
+        bool bnd;
+        const int c = cat_copies<N>(q, dd, idx, bnd);
+        if (!bnd) sum_copies(w, idx, c);
     }
 }
 
@@ -229,10 +266,7 @@ nb_status launch_mask_sc(nb_ctx *c, double *w, const CgScalars *sc) {
         const int grid = grid_blocks(c->m.npts, threads, sm_count() * 8);
         mask_array_kernel<<<grid, threads, 0, c->stream>>>(w, c->m, c->d_mask, sc);
     } else {
-        const Mesh &m = c->m;
-        const int64_t total = 2 * (int64_t)m.n * m.n * ((int64_t)m.ey * m.ez + (int64_t)m.ex * m.ez +
-                                                        (int64_t)m.ex * m.ey);
-        const int grid = grid_blocks(total, threads, sm_count() * 8);
+        const int grid = grid_blocks(box_face_points(c->m), threads, sm_count() * 8);
         mask_box_kernel<<<grid, threads, 0, c->stream>>>(w, c->m, sc);
     }
     NB_LAUNCH_CHECK("mask_kernel");
@@ -243,6 +277,29 @@ nb_status launch_dssum(nb_ctx *c, double *w, bool with_mask) {
     nb_status s = launch_dssum_sc(c, w, nullptr);
     if (s != NB_OK || !with_mask) return s;
     return launch_mask_sc(c, w, nullptr);
+}
+
+// dssum and mask: one launch where the mask is the box's own and there are
+// nodes to share (and the loop's index fits an int).
+nb_status launch_apply_tail(nb_ctx *c, double *w) {
+    int cx, cy, cz;
+    shared_counts(c->m, cx, cy, cz);
+    const int64_t nodes = (int64_t)cx + cy + cz, total = nodes + box_face_points(c->m);
+    if (c->d_mask || nodes == 0 || total > 0x7fffffff - (1 << 24)) return launch_dssum(c, w, true);
+    LaunchTimer tm(c, NB_K_DSSUM);
+    const DsCat dd = make_ds_cat(c->m);
+    const int grid = grid_blocks(total, 256, sm_count() * 5);
+    switch (c->m.n) {
+#define NB_CASE(NN) \
+    case NN: dssum_mask_kernel<NN><<<grid, 256, 0, c->stream>>>(w, dd, c->m); break;
+        NB_CASE(2) NB_CASE(3) NB_CASE(4) NB_CASE(5) NB_CASE(6) NB_CASE(7) NB_CASE(8)
+        NB_CASE(9) NB_CASE(10) NB_CASE(11) NB_CASE(12) NB_CASE(13) NB_CASE(14) NB_CASE(15)
+        NB_CASE(16)
+#undef NB_CASE
+        default: break;
+    }
+    NB_LAUNCH_CHECK("dssum_mask_kernel");
+    return NB_OK;
 }
 
 nb_status launch_mask(nb_ctx *c, double *w) { return launch_mask_sc(c, w, nullptr); }

@@ -85,20 +85,23 @@ __device__ __forceinline__ void divmod(unsigned q, const FastDiv &f, unsigned &q
 }
 
 // Copies of shared node q (a global enumeration over the seven ranges of
-// DsCat) in ascending element order; returns the copy count (2, 4 or 8).
+// DsCat) in ascending element order; returns the copy count (2, 4 or 8).  bnd:
+// the node lies on a face of the box.
 template <int N>
-__device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
+__device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx, bool &bnd) {
     constexpr int N1 = N - 1, N2 = N * N;
     constexpr int64_t N3 = (int64_t)N * N * N;
     const int64_t sy = d.ex, sz = (int64_t)d.ex * d.ey;   // element id strides
     unsigned t, r0, r1;
     int ex, ey, ez, lx, ly, lz;
+    auto end = [](unsigned r, int np) { return r == 0u || r + 1u == (unsigned)np; };
     if (q < d.o[3]) {                         // face nodes: 2 copies
         if (q < d.o[1]) {                     // x-interface a+1 between elements a and a+1
             divmod((unsigned)q, d.fNYp, t, r0);
             divmod(t, d.fNZp, t, r1);
             nonplane_elem<N>((int)r0, d.ey, ey, ly);
             nonplane_elem<N>((int)r1, d.ez, ez, lz);
+            bnd = end(r0, d.NYp) || end(r1, d.NZp);
             const int64_t e = (int64_t)t + sy * ey + sz * ez;
             idx[0] = e * N3 + N1 + N * ly + N2 * lz;
             idx[1] = idx[0] + N3 - N1;
@@ -107,6 +110,7 @@ __device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
             divmod(t, d.fNZp, t, r1);
             nonplane_elem<N>((int)r0, d.ex, ex, lx);
             nonplane_elem<N>((int)r1, d.ez, ez, lz);
+            bnd = end(r0, d.NXp) || end(r1, d.NZp);
             const int64_t e = ex + sy * (int64_t)t + sz * ez;
             idx[0] = e * N3 + lx + N * N1 + N2 * lz;
             idx[1] = idx[0] + sy * N3 - N * N1;
@@ -115,6 +119,7 @@ __device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
             divmod(t, d.fNYp, t, r1);
             nonplane_elem<N>((int)r0, d.ex, ex, lx);
             nonplane_elem<N>((int)r1, d.ey, ey, ly);
+            bnd = end(r0, d.NXp) || end(r1, d.NYp);
             const int64_t e = ex + sy * ey + sz * (int64_t)t;
             idx[0] = e * N3 + lx + N * ly + N2 * N1;
             idx[1] = idx[0] + sz * N3 - N2 * N1;
@@ -128,6 +133,7 @@ __device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
             divmod((unsigned)(q - d.o[3]), d.fNZp, t, r0);
             divmod(t, d.fEx1, t, r1);         // r1 = a, t = b
             nonplane_elem<N>((int)r0, d.ez, ez, lz);
+            bnd = end(r0, d.NZp);
             e = (int64_t)r1 + sy * (int64_t)t + sz * ez;
             l0 = N1 + N * N1 + N2 * lz;
             s1 = 1; s2 = sy;
@@ -139,6 +145,7 @@ __device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
             divmod((unsigned)(q - d.o[4]), d.fNYp, t, r0);
             divmod(t, d.fEx1, t, r1);         // r1 = a, t = c
             nonplane_elem<N>((int)r0, d.ey, ey, ly);
+            bnd = end(r0, d.NYp);
             e = (int64_t)r1 + sy * ey + sz * (int64_t)t;
             l0 = N1 + N * ly + N2 * N1;
             s1 = 1; s2 = sz;
@@ -150,6 +157,7 @@ __device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
             divmod((unsigned)(q - d.o[5]), d.fNXp, t, r0);
             divmod(t, d.fEy1, t, r1);         // r1 = b, t = c
             nonplane_elem<N>((int)r0, d.ex, ex, lx);
+            bnd = end(r0, d.NXp);
             e = ex + sy * (int64_t)r1 + sz * (int64_t)t;
             l0 = lx + N * N1 + N2 * N1;
             s1 = sy; s2 = sz;
@@ -161,6 +169,7 @@ __device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
         return 4;
     }
     // vertices: 8 copies, z outer, y, x inner
+    bnd = false;
     divmod((unsigned)(q - d.o[6]), d.fEx1, t, r0);   // r0 = a
     divmod(t, d.fEy1, t, r1);                          // r1 = b, t = c
     const int64_t e = (int64_t)r0 + sy * (int64_t)r1 + sz * (int64_t)t;
@@ -175,6 +184,12 @@ __device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
     return 8;
 }
 
+
+template <int N>
+__device__ __forceinline__ int cat_copies(int q, const DsCat &d, int64_t *idx) {
+    bool bnd;
+    return cat_copies<N>(q, d, idx, bnd);
+}
 
 // ------------------------------------------------ first copy + fixed offsets
 // The same enumeration as cat_copies, one category at a time, returning only

@@ -193,6 +193,7 @@ nb_status launch_ax(nb_ctx *c, const double *u, double *w);
 nb_status launch_ax_cg(nb_ctx *c);
 // gather-scatter (gs.cu)
 nb_status launch_dssum(nb_ctx *c, double *w, bool with_mask);
+nb_status launch_apply_tail(nb_ctx *c, double *w);   // dssum and mask, one launch where possible
 nb_status launch_mask(nb_ctx *c, double *w);
 nb_status launch_scatter_unique(nb_ctx *c, const double *g, double *loc);
 nb_status launch_tables(nb_ctx *c, int64_t *gid, int32_t *mult, uint8_t *mask);
