@@ -79,11 +79,44 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kAsmThreads, 5)
 assemble_update_kernel(T *__restrict__ r, const T *__restrict__ w, Mesh m, DsCat dd, CgScalars *sc,
                        double *partials, double *hist) {
-    if (sc->done) return;
     constexpr bool F32 = std::is_same<T, float>::value;
     constexpr int N3 = N * N * N;
+    // element-interior points: each step takes UE elements (KI points of
+    // each for this thread) and issues the loads of CH points before their
+    // updates, so up to 2 CH loads are in flight per thread
+    constexpr int NI = N - 2, NI3 = NI > 0 ? NI * NI * NI : 1, ND = NI > 0 ? NI : 1;
+    constexpr int KI = (NI3 + kAsmThreads - 1) / kAsmThreads;
+    constexpr int UE = KI >= 4 ? 1 : 4 / KI, NB = UE * KI, CH = F32 ? 6 : 4;
+    int qk[KI];
+    bool ok[KI];
+    T wv[CH], rv[CH];
+    auto load = [&](int64_t e, int j0) {
+#pragma unroll
+        for (int jj = 0; jj < CH; jj++) {
+            const int j = j0 + jj, u = j / KI, k = j % KI;
+            const int64_t eu = e + (int64_t)u * gridDim.x, q = eu * N3 + qk[k];
+            if (j < NB && ok[k] && eu < m.E) {
+                wv[jj] = __ldcs(w + q);
+                rv[jj] = r[q];
+            }
+        }
+    };
+    // the first step's loads do not wait for the scalars (a solve that is
+    // done has read them for nothing)
+    const int done = sc->done;
     const T alpha = (T)sc->alpha;
     const int erb = (int)((__double_as_longlong(sc->rr) >> 52) & 0x7ff);
+    if constexpr (N > 2) {
+#pragma unroll
+        for (int k = 0; k < KI; k++) {
+            const int qi = threadIdx.x + k * kAsmThreads;
+            const int a = qi % ND, b = (qi / ND) % ND, c = qi / (ND * ND);
+            qk[k] = (1 + a) + N * (1 + b) + N * N * (1 + c);
+            ok[k] = KI * kAsmThreads == NI3 || qi < NI3;
+        }
+        load(blockIdx.x, 0);
+    }
+    if (done) return;
     const int sh = erb == 0 ? 0 : -((erb - 1023) >> 1);
     dfa::SqAcc32 sq;
     dfa::Acc32 acc32;
@@ -95,44 +128,18 @@ assemble_update_kernel(T *__restrict__ r, const T *__restrict__ w, Mesh m, DsCat
             sq.add_sq(v.x, v.y, 1.f);
         }
     };
-    // element-interior points: each step takes UE elements (KI points of
-    // each for this thread) and issues the loads of CH points before their
-    // updates, so up to 2 CH loads are in flight per thread
     if constexpr (N > 2) {
-        constexpr int NI = N - 2, NI3 = NI * NI * NI;
-        constexpr int KI = (NI3 + kAsmThreads - 1) / kAsmThreads;
-        constexpr int UE = KI >= 4 ? 1 : 4 / KI, NB = UE * KI, CH = F32 ? 6 : 4;
-        int qk[KI];
-        bool ok[KI];
-#pragma unroll
-        for (int k = 0; k < KI; k++) {
-            const int qi = threadIdx.x + k * kAsmThreads;
-            const int a = qi % NI, b = (qi / NI) % NI, c = qi / (NI * NI);
-            qk[k] = (1 + a) + N * (1 + b) + N * N * (1 + c);
-            ok[k] = KI * kAsmThreads == NI3 || qi < NI3;
-        }
         for (int64_t e = blockIdx.x; e < m.E; e += (int64_t)UE * gridDim.x) {
 #pragma unroll
             for (int j0 = 0; j0 < NB; j0 += CH) {
-                T wv[CH], rv[CH];
-                int64_t qa[CH];
-                bool go[CH];
+                if (j0 > 0 || e != blockIdx.x) load(e, j0);
 #pragma unroll
                 for (int jj = 0; jj < CH; jj++) {
                     const int j = j0 + jj, u = j / KI, k = j % KI;
                     const int64_t eu = e + (int64_t)u * gridDim.x;
-                    go[jj] = j < NB && ok[k] && eu < m.E;
-                    qa[jj] = eu * N3 + qk[k];
-                    if (go[jj]) {
-                        wv[jj] = __ldcs(w + qa[jj]);
-                        rv[jj] = r[qa[jj]];
-                    }
-                }
-#pragma unroll
-                for (int jj = 0; jj < CH; jj++) {
-                    if (go[jj]) {
+                    if (j < NB && ok[k] && eu < m.E) {
                         const T rn = fma(-alpha, wv[jj], rv[jj]);
-                        r[qa[jj]] = rn;
+                        r[eu * N3 + qk[k]] = rn;
                         add_sq(rn);
                     }
                 }

@@ -129,14 +129,34 @@ dot_kernel(const double *__restrict__ a, const double *__restrict__ b, double *_
     }
 }
 
+// Values of the first two points of a thread in one element, loaded ahead.
+template <int N, bool PRE>
+struct UpdateAhead {
+    static constexpr int K = (N * N * N + kRedThreads - 1) / kRedThreads, C = K < 2 ? K : 2;
+    double w[C], r[C], z[PRE ? C : 1];
+    __device__ __forceinline__ void load(const double *pr, const double *pw, const double *pz) {
+#pragma unroll
+        for (int k = 0; k < C; k++) {
+            const int q = threadIdx.x + k * kRedThreads;
+            if (K * kRedThreads == N * N * N || q < N * N * N) {
+                w[k] = __ldcs(pw + q);
+                r[k] = pr[q];
+                if (PRE) z[k] = pz[q];
+            }
+        }
+    }
+};
+
 // Body of the update: r -= alpha w over this CTA's elements, accumulating
 // <r,r>_c and, with PRE, <r, minv r>_c (shared nodes weighted 1/multiplicity).
+// `ahead` holds the first element's first points; the next element's are
+// loaded after the current one's.
 template <int N, bool PRE>
 __device__ __forceinline__ void update_body(double *__restrict__ r, const double *__restrict__ w, const Mesh &m,
                                             double alpha, const double *__restrict__ minv, double &acc,
-                                            double &accz, int sh) {
+                                            double &accz, int sh, UpdateAhead<N, PRE> &ahead) {
     constexpr int N3 = N * N * N;
-    constexpr int K = (N3 + kRedThreads - 1) / kRedThreads;   // points per thread per element
+    constexpr int K = UpdateAhead<N, PRE>::K;   // points per thread per element
     dfa::SqAcc32 sq;
     unsigned pf[K];
 #pragma unroll
@@ -153,12 +173,14 @@ __device__ __forceinline__ void update_body(double *__restrict__ r, const double
         for (int k = 0; k < K; k++) {
             const int q = threadIdx.x + k * kRedThreads;
             if (K * kRedThreads != N3 && q >= N3) break;
-            const double rn = fma(-alpha, __ldcs(w + base + q), r[base + q]);
+            const bool have = k < UpdateAhead<N, PRE>::C;
+            const int ka = have ? k : 0;
+            const double rn = fma(-alpha, have ? ahead.w[ka] : __ldcs(w + base + q), have ? ahead.r[ka] : r[base + q]);
             r[base + q] = rn;
             const int lg = __popc(pf[k] & sf);
             if (PRE) {
                 acc = fma(scale_down_pow2(rn, lg), rn, acc);
-                accz = fma(scale_down_pow2(rn * minv[base + q], lg), rn, accz);
+                accz = fma(scale_down_pow2(rn * (have ? ahead.z[ka] : minv[base + q]), lg), rn, accz);
             } else {
                 // <r,r>_c on the FP32 pipes: r 2^sh split into a pair with
                 // integer operations, squares accumulated compensated
@@ -166,6 +188,8 @@ __device__ __forceinline__ void update_body(double *__restrict__ r, const double
                 sq.add_sq(v.x, v.y, __uint_as_float((127u - (unsigned)lg) << 23));
             }
         }
+        const int64_t nb = base + (int64_t)gridDim.x * N3;
+        if (e + gridDim.x < m.E) ahead.load(r + nb, w + nb, PRE ? minv + nb : nullptr);
     }
     if (!PRE) acc = sq.value() * __longlong_as_double((long long)(1023 - 2 * sh) << 52);
 }
@@ -177,15 +201,21 @@ template <int N, bool PRE>
 __global__ void __launch_bounds__(kRedThreads, 6)
 update_kernel(double *__restrict__ r, const double *__restrict__ w, Mesh m, double *partials,
               CgScalars *sc, double *hist, const double *__restrict__ minv) {
-    if (sc->done) return;
+    // the first loads do not wait for the scalars (a solve that is done has
+    // read them for nothing)
+    const int done = sc->done;
     const double alpha = sc->alpha;
+    const int erb = (int)((__double_as_longlong(sc->rr) >> 52) & 0x7ff);
+    UpdateAhead<N, PRE> ahead;
+    const int64_t b0 = (int64_t)blockIdx.x * N * N * N;
+    if (blockIdx.x < m.E) ahead.load(r + b0, w + b0, PRE ? minv + b0 : nullptr);
+    if (done) return;
     double acc = 0.0, accz = 0.0, rr, rho;
     // scale 2^sh with (r 2^sh)^2 of order one: from the previous <r,r>_c
     // (the residual changes by modest factors per iteration; the FP32
     // range leaves 2^+-60 of room either way)
-    const int erb = (int)((__double_as_longlong(sc->rr) >> 52) & 0x7ff);
     const int sh = erb == 0 ? 0 : -((erb - 1023) >> 1);
-    update_body<N, PRE>(r, w, m, alpha, minv, acc, accz, sh);
+    update_body<N, PRE>(r, w, m, alpha, minv, acc, accz, sh, ahead);
     if (PRE) {
         double v[2] = {acc, accz}, tot[2];
         if (!last_block_reduce<2>(v, partials, gridDim.x, blockIdx.x, gridDim.x, gridDim.x, &sc->ticket, tot))

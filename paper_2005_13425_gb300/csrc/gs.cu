@@ -23,31 +23,32 @@ namespace nekgb {
 // the first add is a sign fix-up done with integer operations; the remaining
 // adds are exact-count loops (no predicated-off FP64 adds on GB300's narrow
 // FP64 pipe).
+template <typename T, int C>
+__device__ __forceinline__ void sum_copies(T *w, const int64_t *idx, const T (&a)[8]) {
+    T s = plus_zero(a[0]);
+#pragma unroll
+    for (int k = 1; k < C; k++) s = s + a[k];
+#pragma unroll
+    for (int k = 0; k < C; k++) w[idx[k]] = s;
+}
 template <typename T>
-__device__ __forceinline__ void sum_copies(T *w, const int64_t *idx, int c) {
-    if (c == 2) {
-        const T s = plus_zero(w[idx[0]]) + w[idx[1]];
-        w[idx[0]] = s;
-        w[idx[1]] = s;
-    } else if (c == 4) {
-        T a[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) a[k] = w[idx[k]];
-        T s = plus_zero(a[0]);
-#pragma unroll
-        for (int k = 1; k < 4; k++) s = s + a[k];
-#pragma unroll
-        for (int k = 0; k < 4; k++) w[idx[k]] = s;
-    } else {
-        T a[8];
-#pragma unroll
-        for (int k = 0; k < 8; k++) a[k] = w[idx[k]];
-        T s = plus_zero(a[0]);
-#pragma unroll
-        for (int k = 1; k < 8; k++) s = s + a[k];
-#pragma unroll
-        for (int k = 0; k < 8; k++) w[idx[k]] = s;
+__device__ __forceinline__ void load_copies(const T *w, const int64_t *idx, int c, T (&a)[8]) {
+    a[0] = w[idx[0]];
+    a[1] = w[idx[1]];
+    if (c >= 4) {
+        a[2] = w[idx[2]];
+        a[3] = w[idx[3]];
     }
+    if (c == 8) {
+#pragma unroll
+        for (int k = 4; k < 8; k++) a[k] = w[idx[k]];
+    }
+}
+template <typename T>
+__device__ __forceinline__ void sum_copies(T *w, const int64_t *idx, int c, const T (&a)[8]) {
+    if (c == 2) sum_copies<T, 2>(w, idx, a);
+    else if (c == 4) sum_copies<T, 4>(w, idx, a);
+    else sum_copies<T, 8>(w, idx, a);
 }
 
 // Plain dssum (CG = false) or the fused solver step (CG = true), over the
@@ -60,12 +61,24 @@ __device__ __forceinline__ void sum_copies(T *w, const int64_t *idx, int c) {
 template <typename T, bool CG, int N>
 __global__ void __launch_bounds__(256, 5)
 dssum_kernel(T *__restrict__ w, DsCat dd, CgScalars *sc, double *partials, int slot0) {
-    if (sc && sc->done) return;
-    const int total = dd.o[7];
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
-        int64_t idx[8];
-        const int c = cat_copies<N>(q, dd, idx);
-        sum_copies(w, idx, c);
+    // a thread's first node is loaded before the solver's state is known (a
+    // solve that is done has read it for nothing)
+    const int done = sc ? sc->done : 0;
+    const int total = dd.o[7], step = gridDim.x * blockDim.x;
+    int q = blockIdx.x * blockDim.x + threadIdx.x, c = 0;
+    int64_t idx[8];
+    T a[8];
+    auto load = [&]() {
+        if (q >= total) return;
+        c = cat_copies<N>(q, dd, idx);
+        load_copies(w, idx, c, a);
+    };
+    load();
+    if (done) return;
+    while (q < total) {
+        sum_copies(w, idx, c, a);
+        q += step;
+        load();
     }
     if (CG) {
         double v[1] = {0.0}, tot[1];
@@ -149,8 +162,11 @@ dssum_mask_kernel(double *__restrict__ w, DsCat dd, Mesh m) {
         }
         int64_t idx[8];
         bool bnd;
+        double a[8];
         const int c = cat_copies<N>(q, dd, idx, bnd);
-        if (!bnd) sum_copies(w, idx, c);
+        if (bnd) continue;
+        load_copies(w, idx, c, a);
+        sum_copies(w, idx, c, a);
     }
 }
 
