@@ -108,15 +108,15 @@ nb_status prepare_fx(nb_ctx *c) {
     c->d_eo = centro_antisymmetric(c->D_host, c->m.n);
     const int64_t ng = (int64_t)6 * c->m.n * c->m.n * c->m.n * c->m.E;
     const bool df = c->d_eo && df_head_elements(c->m.E, c->m.n);
-    // one allocation: the pairs, the float pairs (few elements) and the exponents
-    const size_t bytes = sizeof(int2) * ng * (df ? 2 : 1) + sizeof(int) * c->m.E;
+    // one allocation: the pairs, the float pairs (few elements), the exponents
+    // and the largest one of the whole box
+    const size_t bytes = sizeof(int2) * ng * (df ? 2 : 1) + sizeof(int) * (c->m.E + 1);
     cudaError_t e = dev_alloc((void **)&c->d_gxyz_fx, bytes);
     if (e != cudaSuccess) return cuda_fail(e, "alloc gxyz pairs");
     c->device_bytes += bytes;
     if (df) c->d_gxyz_df = (float2 *)((int2 *)c->d_gxyz_fx + ng);
     c->d_ge = (int *)((int2 *)c->d_gxyz_fx + ng * (df ? 2 : 1));
-    int *d_ex = nullptr;
-    if ((e = dev_alloc((void **)&d_ex, sizeof(int))) != cudaSuccess) return cuda_fail(e, "alloc exponent");
+    int *d_ex = c->d_ge + c->m.E;
     int gexp = 0;
     const FxRows rows = fx_rows(fx_scales(c->D_host, c->m.n));
     e = cudaMemsetAsync(d_ex, 0, sizeof(int), c->stream);
@@ -129,7 +129,6 @@ nb_status prepare_fx(nb_ctx *c) {
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&gexp, d_ex, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(d_ex);
     if (e != cudaSuccess) return cuda_fail(e, "gxyz pairs");
     gexp = gexp < 1 ? 1 : (gexp > 2046 ? 2046 : gexp);
     c->gxyz_exp = gexp;
