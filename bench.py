@@ -583,30 +583,30 @@ def run_gpu(args, rank, world, local):
     ax_avg_ms = ax["ms_avg"]
     ax_bytes = metrics.cg_head_bytes_per_point(8) * D
     variant = nekgb.nb_get_info(ctx)["ax_variant"]
-    double_float = variant in (0, 2)      # automatic selection picks the double-float kernel at n = 10
+    fixed_point = variant in (0, 2)       # automatic selection picks the fixed-point kernel
     ach_gbs = ax_bytes / (ax_avg_ms * 1e-3) / 1e9
     hbm_frac = ach_gbs / hbm
     total_kernel_ms = sum(v["est_ms"] for v in kern.values())
     traffic = None
-    if double_float:
+    if fixed_point:
         traffic = metrics.recorded_traffic(
-            os.path.join(ROOT, "profiles", "traffic.json"), "cg_head_ax_df_e4096_n10",
+            os.path.join(ROOT, "profiles", "traffic.json"), "cg_head_ax_fx_e4096_n10",
             metrics.source_digest(os.path.join(ROOT, "paper_2005_13425_gb300", "csrc")))
     roof_hbm = {"bound": "hbm", "achieved": ach_gbs, "peak": hbm, "unit": "GB/s",
                 "frac": hbm_frac, "traffic": traffic,
                 "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs, of {peak_src})",
                 "kernel": "ax_e (CG head)", "algorithmic_bytes_per_launch": ax_bytes,
                 "avg_launch_ms": ax_avg_ms, "launches": ax["launches_timed"]}
-    if double_float:
-        # the double-float ax_e runs on the FP32 pipe: its ALU bound is the
-        # FP32 instruction rate, its work the algorithm's FP32 instructions
-        ops = metrics.df_fp32_ops_per_point(NGLL) * D
+    if fixed_point:
+        # the fixed-point ax_e runs on the integer and FP32 pipes: its ALU bound
+        # is the instruction rate, its work the algorithm's multiply-adds
+        ops = metrics.fx_instr_per_point(NGLL) * D
         ach = ops / (ax_avg_ms * 1e-3) / 1e12
         roof_alu = {"bound": "alu", "achieved": ach, "peak": fp32_peak,
-                    "unit": "T FP32 instr/s", "frac": ach / fp32_peak, "traffic": traffic,
+                    "unit": "T instr/s", "frac": ach / fp32_peak, "traffic": traffic,
                     "peak_source": "measured: nb_fp32_rate (FFMA rate, all SMs, this run); nominal "
                                    f"152 SMs x 128 lanes x 2070 MHz = {metrics.FP32_PEAK_TOPS:.2f}",
-                    "kernel": "ax_e (CG head)", "algorithmic_fp32_instr_per_launch": ops,
+                    "kernel": "ax_e (CG head)", "algorithmic_instr_per_launch": ops,
                     "avg_launch_ms": ax_avg_ms, "launches": ax["launches_timed"]}
     else:
         ach = metrics.ax_flops_per_point(NGLL) * D / (ax_avg_ms * 1e-3) / 1e12

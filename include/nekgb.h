@@ -442,8 +442,8 @@ nb_status nb_axpby(nb_ctx *ctx, double alpha, const double *x_dev, double beta,
 /* Measured FP32 instruction rate of the current device (FFMA per second,
  * all SMs, 16 independent chains per thread, best of 5 timed runs after a
  * warm-up; about 30 ms).  The paper has no counterpart: its roofline is
- * bandwidth-only (Sec. V, Eq. 2).  This is the ceiling of the double-float
- * ax_e, whose work is FP32 instructions.  Allocates and frees a small
+ * bandwidth-only (Sec. V, Eq. 2).  This is the instruction ceiling of
+ * ax_e on the integer and FP32 pipes.  Allocates and frees a small
  * scratch buffer and a private stream; synchronous. */
 nb_status nb_fp32_rate(double *ffma_per_s);
 

@@ -2,7 +2,7 @@
 // Listing 1 (arXiv 2005.13425, Sec. III) with FP32 u, w and gxyz, which
 // halves the operator's bytes (32 B per point instead of 64).
 //
-// Same line-thread layout as the double-float kernel (ax_df.cu): 3n^2
+// Same line-thread layout as the double-float head (ax_df.cu): 3n^2
 // threads own one 1-D line each; D entries are compile-time-indexed kernel
 // parameters (constant-bank operands); a pointwise pass contracts with the
 // six geometric factors; the transposed derivatives go to three partial

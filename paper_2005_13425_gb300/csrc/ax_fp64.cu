@@ -12,7 +12,7 @@
 // sum_l dxtm1 * (ur, us, ut), with FP64 fused multiply-adds.
 //
 // GB300 executes FP64 at ~1 TFLOP/s (measured), so this kernel is bound by
-// the FP64 pipe, not by HBM; the double-float kernel (ax_df.cu) is the fast
+// the FP64 pipe, not by HBM; the fixed-point kernel (ax_fx_kernel.cuh) is the fast
 // FP64-accurate path.  This one is kept as the plain-arithmetic variant.
 #include "internal.cuh"
 #include "reduce.cuh"

@@ -1,6 +1,6 @@
 // Measured FP32 instruction rate of the GPU, the denominator of the ALU
-// roofline of the double-float operator (whose work is FP32 instructions:
-// FADD, FMUL and FFMA issue at the same rate on the FMA pipes).
+// roofline of the operator on the integer and FP32 pipes (an upper bound there:
+// FADD, FMUL and FFMA issue at this rate, 64-bit integer multiply-adds slower).
 //
 // Every SM runs its full complement of threads; each thread carries 16
 // independent FFMA chains, so neither dependency latency nor occupancy

@@ -73,7 +73,7 @@ struct ProbDesc {
 
 // ---------------------------------------------------------------- kernels
 // The FP64 CG head on one tile (elements e0 .. e1-1 of problem P): the
-// single-problem head's element loop (ax_df.cu, cg_head_pipelined) over the
+// single-problem head's element loop (ax_df.cu) over the
 // tile's consecutive elements.  The pairs of p are scaled by one power of
 // two per problem and iteration, 2^sh with sqrt(<p,p>_c) 2^sh in [1, 2)
 // (<p,p>_c carried by eng_assemble), so no element needs an exponent scan;

@@ -61,6 +61,17 @@ def df_fp32_ops_per_point(n: int) -> float:
     return lines + contraction + 2 * _ADD + 2
 
 
+def fx_instr_per_point(n: int) -> float:
+    """Multiply-add instructions per point of the fixed-point ax_e (fx.cuh:
+    one 64-bit integer multiply-add and two FFMA per term): 6 even-odd line
+    products of n/2 terms per output (odd n: the pairs of outputs take one
+    middle term more between them, the middle output (n + 1)/2) and the 9
+    terms of the geometric contraction."""
+    h = n // 2
+    terms = h * 2 * h if n % 2 == 0 else h * (2 * h + 1) + h + 1
+    return 3 * (6 * terms / n + 9)
+
+
 def cg_flops_per_point(n: int) -> int:
     """Eq. 1: flops per degree of freedom per CG iteration."""
     return 12 * n + 34
@@ -113,7 +124,7 @@ def measured_peaks(root: str):
         return FALLBACK_HBM_GBS, FALLBACK_BF16_TFLOPS, "fallback"
 
 
-# Sources of the double-float CG head kernel; a recorded DRAM traffic figure
+# Sources of the CG head kernel; a recorded DRAM traffic figure
 # is valid only for the sources it was measured on.
 CG_HEAD_SOURCES = ("ax_fx_kernel.cuh", "ax_fx_core.cuh", "fx.cuh", "reduce.cuh")
 
