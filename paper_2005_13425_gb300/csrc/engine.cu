@@ -1447,6 +1447,14 @@ static nb_status branch_stream(nb_engine *g, int k, cudaStream_t *out) {
     return NB_OK;
 }
 
+// FP64 groups of more elements than this take turns in one branch: a group
+// that fills the GPU by itself loses more by sharing the L2 with another than
+// its tail costs.  100 iterations of
+// FP64 requests at n = 6 to 12, all in turn against all as branches: 232.7 and
+// 221 ms with 7 to 17 thousand elements per group, 309.7 and 305 with 18 to 23,
+// 476.9 and 481 with 22 to 38, 1148 and 1194 with 57 to 91.
+static int64_t branch_elements(const nb_engine *g) { return (int64_t)128 * g->sms; }
+
 // One engine step is a captured graph of `chunk` iterations with one branch per
 // (n, precision): first the outer pass of the mixed requests, then their inner
 // iterations, or the CG iterations of the FP64 requests.  The groups share no
@@ -1463,7 +1471,11 @@ nb_status engine_step_internal(nb_engine *g, int iters) {
     if (s != NB_OK) return s;
     unsigned long long key = 0;
     for (int n = 2; n <= kMaxN; n++) {
-        if (!g->groups[n].slots.empty()) key |= 1ull << n;
+        if (!g->groups[n].slots.empty()) {
+            int64_t elements = 0;
+            for (int slot : g->groups[n].slots) elements += g->h_desc[slot].m.E;
+            key |= (1ull << n) | ((unsigned long long)(elements > branch_elements(g)) << (15 + n));
+        }
         if (!g->mgroups[n].slots.empty()) key |= 1ull << (32 + n);
     }
     if (!key || iters <= 0) return NB_OK;
@@ -1473,9 +1485,12 @@ nb_status engine_step_internal(nb_engine *g, int iters) {
             cudaGraphExecDestroy(g->graph);
             g->graph = nullptr;
         }
-        std::vector<int> order;   // n for FP64 groups, 32 + n for mixed ones
-        for (int b = 0; b < 64; b++)
-            if (key & (1ull << b)) order.push_back(b);
+        std::vector<int> big, order;   // n of FP64 groups, 32 + n of mixed ones
+        for (int n = 2; n <= kMaxN; n++) {
+            if (key & (1ull << n)) (key & (1ull << (15 + n)) ? big : order).push_back(n);
+            if (key & (1ull << (32 + n))) order.push_back(32 + n);
+        }
+        if (!big.empty()) order.insert(order.begin(), 0);   // the big groups' branch
         cudaStream_t br = nullptr;
         for (int k = 0; k < (int)order.size(); k++)   // created outside the capture
             if ((s = branch_stream(g, k, &br)) != NB_OK) return s;
@@ -1489,8 +1504,10 @@ nb_status engine_step_internal(nb_engine *g, int iters) {
             if (k > 0) ef = cudaStreamWaitEvent(br, g->fork, 0);
             g->launch = br;
             if (s == NB_OK && ef == cudaSuccess && mixed) s = dispatch_mixed(g, n, true);
-            for (int it = 0; it < chunk && s == NB_OK && ef == cudaSuccess; it++)
-                s = mixed ? dispatch_mixed(g, n, false) : dispatch_iteration(g, n);
+            for (int it = 0; it < chunk && s == NB_OK && ef == cudaSuccess; it++) {
+                if (n > 0) s = mixed ? dispatch_mixed(g, n, false) : dispatch_iteration(g, n);
+                for (size_t q = 0; n == 0 && q < big.size() && s == NB_OK; q++) s = dispatch_iteration(g, big[q]);
+            }
         }
         for (int k = 1; k < (int)order.size() && s == NB_OK && ef == cudaSuccess; k++) {
             s = branch_stream(g, k, &br);
