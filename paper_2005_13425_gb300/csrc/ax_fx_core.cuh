@@ -319,7 +319,7 @@ __device__ __forceinline__ void fx_operator(const FxThread<N, G> &th, bool on, i
         if (G == 1 || th.d == 0) fx_line_at<N, EO, false, 0>(X + th.line(0), R + th.line(0), D);
         if (G == 1 || th.d == 1) fx_line_at<N, EO, false, 1>(X + th.line(1), S + th.line(1), D);
         if (G == 3 && th.d == 2) fx_line_at<N, EO, false, 2>(X + th.line(2), TT + th.line(2), D);
-        load(0, gb[0]);
+        if (th.has(0)) load(0, gb[0]);     // n = 2 with G = 3: the third thread owns no point
         if (K > 1 && th.has(1)) load(1, gb[1]);
     }
     __syncthreads();
