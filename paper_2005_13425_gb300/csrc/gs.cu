@@ -51,36 +51,68 @@ __device__ __forceinline__ void sum_copies(T *w, const int64_t *idx, int c, cons
     else sum_copies<T, 8>(w, idx, a);
 }
 
-// Plain dssum (CG = false) or the fused solver step (CG = true), over the
-// shared nodes grouped by category (faces, edges, vertices; DsCat).  In the
-// solver the ax_e head has already summed
-// <w,p>_c as local products (p is continuous, so the assembled product
-// equals the sum of the unassembled ones); the last CTA here reduces those
-// partials, forms alpha = rho/<w,p>_c and flags a breakdown.  N is the
-// number of points per direction.
-template <typename T, bool CG, int N>
-__global__ void __launch_bounds__(256, 5)
-dssum_kernel(T *__restrict__ w, DsCat dd, CgScalars *sc, double *partials, int slot0) {
-    // a thread's first node is loaded before the solver's state is known (a
-    // solve that is done has read it for nothing)
-    const int done = sc ? sc->done : 0;
-    const int total = dd.o[7], step = gridDim.x * blockDim.x;
-    int q = blockIdx.x * blockDim.x + threadIdx.x, c = 0;
+// One shared node of the plain dssum: the loads and the sum of a copy count
+// together, so that few values live across the loop's back edge.
+template <typename T, int N>
+__device__ __forceinline__ void sum_node(T *w, int q, const DsCat &dd) {
     int64_t idx[8];
     T a[8];
-    auto load = [&]() {
-        if (q >= total) return;
-        c = cat_copies<N>(q, dd, idx);
-        load_copies(w, idx, c, a);
+    auto sum = [&](auto count) {
+        constexpr int C = decltype(count)::value;
+#pragma unroll
+        for (int k = 0; k < C; k++) a[k] = w[idx[k]];
+        sum_copies<T, C>(w, idx, a);
     };
-    load();
-    if (done) return;
-    while (q < total) {
-        sum_copies(w, idx, c, a);
-        q += step;
+    const int c = cat_copies<N>(q, dd, idx);
+    if (c == 2) sum(std::integral_constant<int, 2>());
+    else if (c == 4) sum(std::integral_constant<int, 4>());
+    else sum(std::integral_constant<int, 8>());
+}
+
+// dssum over the shared nodes grouped by category (faces, edges, vertices;
+// DsCat).
+enum DssumMode {
+    kDssumPlain,    // the call of its own
+    kDssumSolver,   // in a solve: nothing once it is done
+    kDssumCg        // in a solve whose ax_e head has summed <w,p>_c
+};
+// kDssumCg: the head's sum is of the local products (p is continuous, so the
+// assembled product equals the sum of the unassembled ones); the last CTA here
+// reduces those partials, forms alpha = rho/<w,p>_c and flags a breakdown.
+// N is the number of points per direction.
+//
+// In a solve a thread's first node is loaded before the solver's state is known
+// (a solve that is done has read it for nothing), the next one after the
+// current one's stores.  The plain call has no state to wait for, and there the
+// copies that live across the loop cost more than they hide: FP32 12.8 us loaded
+// ahead and 12.4 not (2048 elements at n = 10), FP64 20.55 and 20.5 (4096 at
+// n = 10), 244.8 and 245.9 (32768 at n = 12).
+template <typename T, DssumMode MODE, int N>
+__global__ void __launch_bounds__(256, 5)
+dssum_kernel(T *__restrict__ w, DsCat dd, CgScalars *sc, double *partials, int slot0) {
+    const int total = dd.o[7], step = gridDim.x * blockDim.x;
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if constexpr (MODE == kDssumPlain) {
+        for (; q < total; q += step) sum_node<T, N>(w, q, dd);
+    } else {
+        const int done = sc->done;
+        int c = 0;
+        int64_t idx[8];
+        T a[8];
+        auto load = [&]() {
+            if (q >= total) return;
+            c = cat_copies<N>(q, dd, idx);
+            load_copies(w, idx, c, a);
+        };
         load();
+        if (done) return;
+        while (q < total) {
+            sum_copies(w, idx, c, a);
+            q += step;
+            load();
+        }
     }
-    if (CG) {
+    if constexpr (MODE == kDssumCg) {
         double v[1] = {0.0}, tot[1];
         if (!last_block_reduce<1>(v, partials, 0, slot0 + blockIdx.x, slot0 + gridDim.x, gridDim.x,
                                   &sc->ticket, tot))
@@ -231,13 +263,13 @@ int dssum_grid(const nb_ctx *c) {
     return grid_blocks((int64_t)cx + cy + cz, 256, sm_count() * 5);
 }
 
-template <typename T, bool CG>
+template <typename T, DssumMode MODE>
 static void dssum_launch(nb_ctx *c, T *w, CgScalars *sc, double *partials, int slot0) {
     const DsCat dd = make_ds_cat(c->m);
     const int grid = dssum_grid(c);
     switch (c->m.n) {
 #define NB_CASE(NN) \
-    case NN: dssum_kernel<T, CG, NN><<<grid, 256, 0, c->stream>>>(w, dd, sc, partials, slot0); break;
+    case NN: dssum_kernel<T, MODE, NN><<<grid, 256, 0, c->stream>>>(w, dd, sc, partials, slot0); break;
         NB_CASE(2) NB_CASE(3) NB_CASE(4) NB_CASE(5) NB_CASE(6) NB_CASE(7) NB_CASE(8)
         NB_CASE(9) NB_CASE(10) NB_CASE(11) NB_CASE(12) NB_CASE(13) NB_CASE(14) NB_CASE(15)
         NB_CASE(16)
@@ -251,7 +283,8 @@ nb_status launch_dssum_sc(nb_ctx *c, double *w, const CgScalars *sc) {
     shared_counts(c->m, cx, cy, cz);
     if ((int64_t)cx + cy + cz == 0) return NB_OK;
     LaunchTimer tm(c, NB_K_DSSUM);
-    dssum_launch<double, false>(c, w, const_cast<CgScalars *>(sc), nullptr, 0);
+    if (sc) dssum_launch<double, kDssumSolver>(c, w, const_cast<CgScalars *>(sc), nullptr, 0);
+    else dssum_launch<double, kDssumPlain>(c, w, nullptr, nullptr, 0);
     NB_LAUNCH_CHECK("dssum_kernel");
     return NB_OK;
 }
@@ -259,7 +292,7 @@ nb_status launch_dssum_sc(nb_ctx *c, double *w, const CgScalars *sc) {
 // Fused solver step: dssum of w and alpha = rho/<w,p>_c.
 nb_status launch_dssum_cg(nb_ctx *c) {
     LaunchTimer tm(c, NB_K_DSSUM);
-    dssum_launch<double, true>(c, c->d_w, c->d_sc, c->d_partials, c->ax_grid);
+    dssum_launch<double, kDssumCg>(c, c->d_w, c->d_sc, c->d_partials, c->ax_grid);
     NB_LAUNCH_CHECK("dssum_kernel<cg>");
     return NB_OK;
 }
@@ -270,7 +303,7 @@ nb_status launch_dssum32(nb_ctx *c, float *w) {
     shared_counts(c->m, cx, cy, cz);
     if ((int64_t)cx + cy + cz == 0) return NB_OK;
     LaunchTimer tm(c, NB_K_DSSUM);
-    dssum_launch<float, false>(c, w, nullptr, nullptr, 0);
+    dssum_launch<float, kDssumPlain>(c, w, nullptr, nullptr, 0);
     NB_LAUNCH_CHECK("dssum_kernel<f32>");
     return NB_OK;
 }
