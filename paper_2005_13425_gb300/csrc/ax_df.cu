@@ -31,6 +31,7 @@ struct AxDfArgs {
     double *partials;     // one <w,p> partial per CTA
     int dot_shift0;       // scale of the exact <w,p>_c sum (see launch_df_n)
     int dot_lim;          // a share of 2^dot_lim or more (scaled) may overflow the sum
+    int finite;           // the operator's data (D and gxyz) has no NaN or Inf
     Mesh m;
     const float2 *g;      // gxyz pairs [E][6][n^3], scaled by 2^-(gexp-1023)
     int gexp;             // biased exponent of max|gxyz|
@@ -239,7 +240,7 @@ ax_df_head_kernel(AxDfArgs a, const __grid_constant__ DfEo<N> D) {
     const int S = a.dot_shift0 - ((int)((__double_as_longlong(pn) >> 52) & 0x7ff) - 1023);
     bool out_of_range = false;
     const u128 mine = block_sum_u128(df_head_pipelined<N>(a, beta, xa, S, D, sm, out_of_range), red);
-    finish_exact_sum(a.sc, a.partials, mine, S, out_of_range, red);
+    finish_exact_sum(a.sc, a.partials, mine, S, out_of_range, a.finite && finite_pp(pn), red);
 }
 
 // ---------------------------------------------------------------- set-up
@@ -325,6 +326,7 @@ static nb_status launch_df_n(nb_ctx *c) {
     args.partials = c->d_partials;
     args.dot_shift0 = dot_shift0<N>(c) + c->test_dot_shift;
     args.dot_lim = dot_lim<N>(c);
+    args.finite = c->op_finite;
     args.m = c->m;
     auto kern = ax_df_head_kernel<N>;
     {

@@ -118,7 +118,12 @@ nb_status prepare_fx(nb_ctx *c) {
     c->d_ge = (int *)((int2 *)c->d_gxyz_fx + ng * (df ? 2 : 1));
     int *d_ex = c->d_ge + c->m.E;
     int gexp = 0;
-    const FxRows rows = fx_rows(fx_scales(c->D_host, c->m.n));
+    bool d_finite = true;
+    for (int q = 0; q < c->m.n * c->m.n; q++) d_finite = d_finite && isfinite(c->D_host[q]);
+    FxRows rows = fx_rows(fx_scales(c->D_host, c->m.n));
+    // a D that is not finite has no fixed-point form: every element's factors
+    // become "not finite" (and so its results), and the tables stay 0
+    for (int i = 0; i < kMaxN && !d_finite; i++) rows.rho[i] = NAN;
     e = cudaMemsetAsync(d_ex, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) {
         const int64_t cap = (int64_t)device_sms() * 8;
@@ -130,11 +135,12 @@ nb_status prepare_fx(nb_ctx *c) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(&gexp, d_ex, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "gxyz pairs");
+    c->op_finite = d_finite && gexp < 2047;
     gexp = gexp < 1 ? 1 : (gexp > 2046 ? 2046 : gexp);
     c->gxyz_exp = gexp;
     fx_tables(c);
     c->fx_dot_lim = fx_dot_lim(c);
-    c->fx_dot_shift0 = fx_dot_shift0(c);
+    c->fx_dot_shift0 = c->op_finite ? fx_dot_shift0(c) : 0;
     return df ? prepare_df(c) : NB_OK;
 }
 

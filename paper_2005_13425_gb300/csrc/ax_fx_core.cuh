@@ -429,7 +429,7 @@ __device__ __forceinline__ unsigned fx_top_of(const FxThread<N, G> &th, const do
 }
 __device__ __forceinline__ int fx_emax(unsigned top) {
     const int e = (int)(top >> 20);
-    return e < fx::kMinExp ? fx::kMinExp : e;
+    return e < fx::kMinExp ? fx::kMinExp : (e == 0x7ff ? fx::kNotFinite : e);
 }
 __device__ __forceinline__ int2 fx_input(double v, int emax) {
     const fx::Pair p = fx::from_double(v, emax);
@@ -640,7 +640,7 @@ inline FxRows fx_rows(const FxScales &S) {
 // The scale of a point's six scaled factors v (rr, rs, rt, ss, st, tt): the
 // exponent eq with which the largest absolute row sum of the 3 x 3 matrix
 // lies in (2^30, 2^31], in units of 2^(eq - 1053).  ex: the factors' biased
-// exponents (0: the factor counts as 0).
+// exponents (0: the factor counts as 0).  kNotFinite if one of them is NaN or Inf.
 __device__ __forceinline__ int fx_point_exponent(const double (&v)[6], int (&ex)[6]) {
     int e0 = 0;
 #pragma unroll
@@ -648,6 +648,7 @@ __device__ __forceinline__ int fx_point_exponent(const double (&v)[6], int (&ex)
         ex[c] = (int)((__double_as_longlong(v[c]) >> 52) & 0x7ff);
         e0 = ex[c] > e0 ? ex[c] : e0;
     }
+    if (e0 == 0x7ff) return fx::kNotFinite;
     unsigned long long m[6];   // magnitudes rounded up, 31 bits for the largest
 #pragma unroll
     for (int c = 0; c < 6; c++) {

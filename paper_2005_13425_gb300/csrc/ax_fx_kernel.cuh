@@ -36,6 +36,7 @@ struct AxFxArgs {
     double *partials;     // MODE 1 with fuse, MODE 2: one <w,p> partial per CTA
     int dot_shift0;       // MODE 2: scale of the exact <w,p>_c sum (see launch_fx_nv)
     int dot_lim;          // MODE 2: a share of 2^dot_lim or more (scaled) may overflow the sum
+    int finite;           // MODE 2: the operator's data (D and gxyz) has no NaN or Inf
     int fuse;             // MODE 1: zero box-face points, local products w p
     Mesh m;
     const int4 *g;        // gxyz pairs [E][3][n^3], two per entry
@@ -159,7 +160,7 @@ ax_fx_kernel(AxFxArgs a, const __grid_constant__ typename FxConsts<N, EO>::type 
         const int S = a.dot_shift0 - ((int)((__double_as_longlong(pn) >> 52) & 0x7ff) - 1023);
         bool out_of_range = false;
         const u128 mine = block_sum_u128(cg_head_pipelined<N, EO, G>(a, beta, xa, S, D, sm, s_max, out_of_range), red);
-        finish_exact_sum(a.sc, a.partials, mine, S, out_of_range, red);
+        finish_exact_sum(a.sc, a.partials, mine, S, out_of_range, a.finite && finite_pp(pn), red);
     } else {
         FxThread<N, G> th;
         th.init();
@@ -208,6 +209,7 @@ static nb_status launch_fx_nv(nb_ctx *c, const double *u, double *w, int mode) {
         args.fuse = c->fused_cg ? 1 : 0;
         args.dot_shift0 = c->fx_dot_shift0 + c->test_dot_shift;
         args.dot_lim = c->fx_dot_lim;
+        args.finite = c->op_finite;
     }
     args.m = c->m;
     auto kern = mode == 0 ? ax_fx_kernel<N, 0, EO, G> : ax_fx_kernel<N, 1, EO, G>;
@@ -242,6 +244,8 @@ void fx_tables_n(nb_ctx *c) {
         using T = std::remove_pointer_t<decltype(D)>;
         static_assert(sizeof(T) % sizeof(int4) == 0, "");
         c->fx_tab.resize(sizeof(T) / sizeof(int4));
+        for (int q = 0; q < N * N; q++)
+            if (!isfinite(c->D_host[q])) return;   // see prepare_fx
         fx_consts<N, decltype(eo)::value>(c->D_host, *reinterpret_cast<T *>(c->fx_tab.data()));
     };
     if (c->d_eo) make((typename FxConsts<N, true>::type *)nullptr, std::true_type{});

@@ -41,16 +41,22 @@ __device__ __forceinline__ double scale_pow2(double x, int k) {
     return x * __longlong_as_double((long long)(k1 + 1023) << 52) * __longlong_as_double((long long)(k2 + 1023) << 52);
 }
 
+// Is <p,p>_c finite?  The integer sum cannot carry a NaN or an Inf of p, so a head
+// ends the solve when this does not hold (or the operator's data is not finite).
+__device__ __forceinline__ bool finite_pp(double pn) {
+    return (int)((__double_as_longlong(pn) >> 52) & 0x7ff) != 0x7ff;
+}
+
 // The sums of a head's threads (at the scale 2^S) over the CTA, and by the last
 // CTA over all of them; that CTA forms alpha.  Every thread must call it.  red:
 // 32 doubles of shared memory (as many as 2 per warp).
 __device__ __forceinline__ void finish_exact_sum(CgScalars *sc, double *partials, u128 mine, int S, bool out_of_range,
-                                                 double *red) {
+                                                 bool finite, double *red) {
     const int range_fault = __syncthreads_or(out_of_range);
     __shared__ int s_last;
     if (threadIdx.x == 0) {
-        if (range_fault) {           // seen by the last CTA's finalize_alpha, which ends the solve
-            sc->fault = kFaultExactSumRange;
+        if (range_fault || !finite) {   // seen by the last CTA's finalize_alpha, which ends the solve
+            if (finite) sc->fault = kFaultExactSumRange;
             sc->status = (int)NB_ERR_BREAKDOWN;
         }
         partials[2 * blockIdx.x] = __longlong_as_double((long long)(unsigned long long)(mine >> 64));

@@ -108,6 +108,10 @@ __host__ __device__ __forceinline__ Pair pair_of(long long A, float B) {
 // caller's emax is at least kMinExp, so a subnormal v (whose mantissa has no
 // implicit bit) is shifted out.
 constexpr int kMinExp = 64;
+// An exponent that stands for "not finite" (a NaN or an Inf in an element's input
+// or factors), far above every exponent of finite data (below 2^12, as sums of
+// them): its values become 0, and Scale makes the results NaN.
+constexpr int kNotFinite = 1 << 14;
 __host__ __device__ __forceinline__ Pair from_double(double v, int emax) {
     const unsigned long long b = (unsigned long long)d_bits(v);
     const unsigned hi = (unsigned)(b >> 32);
@@ -138,7 +142,8 @@ __host__ __device__ __forceinline__ double scale2(double x, int k) {
 // them and take their offsets off: every step but the last is exact.
 // Outside +-900 (ext) the caller multiplies the results by a second factor,
 // post, which brings the exponent to where it belongs (they then overflow or
-// underflow as FP64 does).
+// underflow as FP64 does).  The same factor makes the results of an element with
+// non-finite data NaN.
 struct Scale {
     double f, f2, c, post;
     bool ext;
@@ -150,7 +155,7 @@ struct Scale {
         ext = s != so;
         s = so - s;
         s = s < -1022 ? -1022 : (s > 1023 ? 1023 : s);
-        post = pow2(s);
+        post = so > kNotFinite / 2 ? bits_d(0x7ff8000000000000ll) : pow2(s);
     }
     __host__ __device__ __forceinline__ double operator()(Pair p) const {
 #ifdef __CUDA_ARCH__

@@ -124,6 +124,7 @@ struct nb_ctx {
     float *d_gxyz32 = nullptr;  // [E][6][n^3] fp32 for the mixed inner solve
     float2 *d_gxyz_df = nullptr;  // [E][6][n^3] float pairs for the CG head on few elements (ax_df.cu; in d_gxyz_fx's allocation), or null
     int gxyz_exp = 1023;        // biased exponent of max|gxyz|
+    bool op_finite = true;      // neither D nor gxyz holds a NaN or an Inf
     bool d_eo = false;          // D is centro-antisymmetric: even-odd line products
     bool is_box = false;        // built by nb_setup_box (coordinates known)
     // slab of a z-partitioned box (nb_setup_slab): element layers
