@@ -33,6 +33,21 @@ struct DfEo {
     EoMat<N> bwd;   // M = D^T
 };
 
+// The plain form, for a matrix that is not centro-antisymmetric.
+template <int N>
+struct DfMat {
+    struct Half {
+        float h[N * N], l[N * N];
+    } fwd, bwd;
+};
+
+template <int N, bool EO>
+struct DfConsts;
+template <int N>
+struct DfConsts<N, false> { using type = DfMat<N>; };
+template <int N>
+struct DfConsts<N, true> { using type = DfEo<N>; };
+
 
 // One line task per thread up to n = 12; two per thread above, so that the
 // n-long line held in registers does not spill at n = 16.
@@ -119,6 +134,36 @@ __device__ __forceinline__ void line_eo(const float2 *in, float2 *out, int base,
         dfa::fma(Y, M.ch[H], M.cl[H], ch, cl);
         out[base + H * stride] = dfa::norm(Y);
     }
+}
+
+// The same in plain form, the outputs as unnormalised pairs.
+template <int N>
+__device__ __forceinline__ void line_plain(const float2 *in, float2 *out, int base, int stride,
+                                           const typename DfMat<N>::Half &M) {
+    float2 x[N];
+#pragma unroll
+    for (int l = 0; l < N; l++) x[l] = in[base + l * stride];
+#pragma unroll 1
+    for (int m = 0; m < N; m++) {
+        dfa::Acc acc = dfa::first(M.h[m * N], M.l[m * N], x[0].x, x[0].y);
+#pragma unroll
+        for (int l = 1; l < N; l++) dfa::fma(acc, M.h[m * N + l], M.l[m * N + l], x[l].x, x[l].y);
+        out[base + m * stride] = dfa::raw(acc);
+    }
+}
+
+// u = g w at one point, in place: g = (rr, rs, rt, ss, st, tt).
+__device__ __forceinline__ void df_contract(const float2 (&g)[6], float2 &a, float2 &b, float2 &c) {
+    auto row = [&](int q0, int q1, int q2) {
+        dfa::Acc u = dfa::first(g[q0].x, g[q0].y, a.x, a.y);
+        dfa::fma(u, g[q1].x, g[q1].y, b.x, b.y);
+        dfa::fma(u, g[q2].x, g[q2].y, c.x, c.y);
+        return dfa::raw(u);
+    };
+    const float2 r = row(0, 1, 2), s = row(1, 3, 4), t = row(2, 4, 5);
+    a = r;
+    b = s;
+    c = t;
 }
 
 // Points of an element per thread of a T-thread CTA in the pointwise phases.
@@ -223,6 +268,24 @@ inline void eo_consts(const double *Dm, bool tr, EoMat<N> &E) {
         }
     }
     for (int l = 0; l <= H; l++) put((N & 1) ? M(H, l) : 0.0, E.ch[l], E.cl[l]);
+}
+
+template <int N, bool EO>
+inline void df_consts(const double *Dm, typename DfConsts<N, EO>::type &C) {
+    if constexpr (EO) {
+        eo_consts<N>(Dm, false, C.fwd);
+        eo_consts<N>(Dm, true, C.bwd);
+    } else {
+        auto put = [](double v, float &h, float &l) {
+            h = (float)v;
+            l = (float)(v - (double)h);
+        };
+        for (int m = 0; m < N; m++)
+            for (int l = 0; l < N; l++) {
+                put(Dm[m * N + l], C.fwd.h[m * N + l], C.fwd.l[m * N + l]);
+                put(Dm[l * N + m], C.bwd.h[m * N + l], C.bwd.l[m * N + l]);
+            }
+    }
 }
 
 }  // namespace nekgb

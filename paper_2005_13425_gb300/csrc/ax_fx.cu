@@ -14,12 +14,17 @@ void fx_tables_n(nb_ctx *c);
 
 // ---------------------------------------------------------------- set-up
 // gxyz in fixed-point pairs (ax_fx_core.cuh, Scales), one CTA per element:
-// first each point's exponent and their maximum ge, then the pairs.
+// first each point's exponent and their maximum ge, then the pairs.  The
+// element's word (ax_fx_core.cuh, Graded elements): kFxGraded if a point's
+// factors lie further below the element's largest than they do on a regular
+// element of this order by 2^5 (measured with Jacobians graded up to 2^18: no
+// larger error than the double-float operator's relative to max|w|, and up to
+// 2^7 times as large relative to the point's own terms), or all_graded.
 __global__ void __launch_bounds__(256)
 fx_factors_kernel(const double *__restrict__ x, int4 *__restrict__ y, int *__restrict__ ge, int64_t E, int n,
-                  FxRows rows) {
+                  FxRows rows, bool all_graded, int *special) {
     const int n3 = n * n * n;
-    __shared__ int s_ge;
+    __shared__ int s_ge, s_low, s_gd[3];
     for (int64_t e = blockIdx.x; e < E; e += gridDim.x) {
         const double *g = x + e * 6 * n3;
         auto point = [&](int q, double (&v)[6], int (&ex)[6]) {
@@ -29,15 +34,26 @@ fx_factors_kernel(const double *__restrict__ x, int4 *__restrict__ y, int *__res
             return fx_point_exponent(v, ex);
         };
         double v[6];
-        int ex[6], top = 0;
+        int ex[6], top = 0, low = 1 << 20, gd[3] = {0, 0, 0};
         __syncthreads();
-        if (threadIdx.x == 0) s_ge = 0;
+        if (threadIdx.x == 0) {
+            s_ge = 0;
+            s_low = 1 << 20;
+            for (int d = 0; d < 3; d++) s_gd[d] = 0;
+        }
         __syncthreads();
         for (int q = threadIdx.x; q < n3; q += blockDim.x) {
             const int eq = point(q, v, ex);
             top = eq > top ? eq : top;
+            if (eq > 0) low = eq < low ? eq : low;      // 0: no factors at all
+            for (int d = 0; d < 3; d++) {
+                const int x = ex[d == 0 ? 0 : 2 * d + 1];
+                gd[d] = x > gd[d] ? x : gd[d];
+            }
         }
         atomicMax(&s_ge, top);
+        atomicMin(&s_low, low);
+        for (int d = 0; d < 3; d++) atomicMax(&s_gd[d], gd[d]);
         __syncthreads();
         top = s_ge;
         for (int q = threadIdx.x; q < n3; q += blockDim.x) {
@@ -47,7 +63,12 @@ fx_factors_kernel(const double *__restrict__ x, int4 *__restrict__ y, int *__res
 #pragma unroll
             for (int c = 0; c < 3; c++) y[(e * 3 + c) * n3 + q] = o[c];
         }
-        if (threadIdx.x == 0) ge[e] = top;
+        if (threadIdx.x == 0) {
+            for (int d = 0; d < 3; d++) gd[d] = s_gd[d];
+            const int word = top | fx_weak_bits(gd) | (all_graded || top - s_low > fx_max_shift(n) ? kFxGraded : 0);
+            ge[e] = word;
+            if (word & kFxSpecial) *special = 1;
+        }
     }
 }
 
@@ -108,37 +129,48 @@ nb_status prepare_fx(nb_ctx *c) {
     c->d_eo = centro_antisymmetric(c->D_host, c->m.n);
     const int64_t ng = (int64_t)6 * c->m.n * c->m.n * c->m.n * c->m.E;
     const bool df = c->d_eo && df_head_elements(c->m.E, c->m.n);
-    // one allocation: the pairs, the float pairs (few elements), the exponents
-    // and the largest one of the whole box
-    const size_t bytes = sizeof(int2) * ng * (df ? 2 : 1) + sizeof(int) * (c->m.E + 1);
+    // one allocation: the pairs, the float pairs (few elements), the elements'
+    // words, the largest exponent of the whole box and whether an element is
+    // special, D in double-float pairs, the scratch of graded elements
+    const size_t bytes = sizeof(int2) * (ng * (df ? 2 : 1) + c->m.E) + sizeof(int) * (c->m.E + 2) +
+                         sizeof(float) * fx_df_floats(c->m.n);
     cudaError_t e = dev_alloc((void **)&c->d_gxyz_fx, bytes);
     if (e != cudaSuccess) return cuda_fail(e, "alloc gxyz pairs");
     c->device_bytes += bytes;
     if (df) c->d_gxyz_df = (float2 *)((int2 *)c->d_gxyz_fx + ng);
-    c->d_ge = (int *)((int2 *)c->d_gxyz_fx + ng * (df ? 2 : 1));
+    c->d_redo_list = (int2 *)c->d_gxyz_fx + ng * (df ? 2 : 1);
+    c->d_ge = (int *)(c->d_redo_list + c->m.E);
     int *d_ex = c->d_ge + c->m.E;
-    int gexp = 0;
+    c->d_D_df = (float *)(d_ex + 2);
+    int found[2] = {0, 0};
     bool d_finite = true;
     for (int q = 0; q < c->m.n * c->m.n; q++) d_finite = d_finite && isfinite(c->D_host[q]);
     FxRows rows = fx_rows(fx_scales(c->D_host, c->m.n));
     // a D that is not finite has no fixed-point form: every element's factors
     // become "not finite" (and so its results), and the tables stay 0
     for (int i = 0; i < kMaxN && !d_finite; i++) rows.rho[i] = NAN;
-    e = cudaMemsetAsync(d_ex, 0, sizeof(int), c->stream);
+    e = cudaMemsetAsync(d_ex, 0, sizeof found, c->stream);
     if (e == cudaSuccess) {
         const int64_t cap = (int64_t)device_sms() * 8;
         max_exponent_kernel<<<1024, 256, 0, c->stream>>>(c->d_gxyz, ng, d_ex);
         fx_factors_kernel<<<(int)(c->m.E < cap ? c->m.E : cap), 256, 0, c->stream>>>(c->d_gxyz, c->d_gxyz_fx, c->d_ge,
-                                                                                c->m.E, c->m.n, rows);
+                                                                                c->m.E, c->m.n, rows,
+                                                                                d_finite && fx_graded_matrix(c->D_host, c->m.n),
+                                                                                d_ex + 1);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&gexp, d_ex, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    fx_tables(c);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->d_D_df, c->df_tab.data(), sizeof(float) * c->df_tab.size(), cudaMemcpyHostToDevice,
+                            c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(found, d_ex, sizeof found, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "gxyz pairs");
+    int gexp = found[0];
+    c->fx_special = found[1];
     c->op_finite = d_finite && gexp < 2047;
     gexp = gexp < 1 ? 1 : (gexp > 2046 ? 2046 : gexp);
     c->gxyz_exp = gexp;
-    fx_tables(c);
     c->fx_dot_lim = fx_dot_lim(c);
     c->fx_dot_shift0 = c->op_finite ? fx_dot_shift0(c) : 0;
     return df ? prepare_df(c) : NB_OK;

@@ -27,6 +27,7 @@
 // (h + l) 2^so with so = emax + ge - k - 2009.
 #pragma once
 
+#include "ax_df_core.cuh"
 #include "fx.cuh"
 #include "internal.cuh"
 #include "reduce.cuh"
@@ -138,6 +139,12 @@ __host__ __device__ constexpr int fx_min_blocks() {
     constexpr int b = by_smem < by_regs ? by_smem : by_regs;
     return b < 1 ? 1 : (b > 24 ? 24 : b);
 }
+
+// Exponents below the element's largest from which entries count as small (see
+// Graded elements).
+__host__ __device__ constexpr int fx_grade(int n) { return n == 2 ? 11 : (n == 3 ? 10 : 8); }
+// Top words of elements that are graded because all their entries are tiny.
+constexpr unsigned kFxTiny = (unsigned)(fx::kMinExp + 1) << 20;
 
 // A thread's place: its element within the CTA's group, (i, j) and, with
 // G = 3, its number d in the column.
@@ -302,13 +309,14 @@ __device__ __forceinline__ void fx_contract(const int4 (&g4)[3], int2 &a, int2 &
 // thread's own column only.  Barriers between phases; none before the first
 // and none after the last.  The pointers are the element's; g: its factors at
 // the thread's column, [3][n^3].  on: the thread has a column of an element.
+// s_low: with G = 3, the word that receives all ones if a t line is small (fx_note).
 // Two points' factors are loaded ahead, the first before the barrier.  The
 // loop over the points is not unrolled further: the straight-line code of an
 // element did not fit the instruction cache.
 template <int N, bool EO, int G>
 __device__ __forceinline__ void fx_operator(const FxThread<N, G> &th, bool on, int2 *X, int2 *R, int2 *S, int2 *TT,
-                                            const int4 *__restrict__ g,
-                                            const typename FxConsts<N, EO>::type &D) {
+                                            const int4 *__restrict__ g, const typename FxConsts<N, EO>::type &D,
+                                            unsigned *s_low) {
     constexpr int N2 = N * N, N3 = N * N * N, L = fx_layer(N), K = FxThread<N, G>::K;
     int4 gb[2][3];
     auto load = [&](int kk, int4 (&b)[3]) {
@@ -318,7 +326,16 @@ __device__ __forceinline__ void fx_operator(const FxThread<N, G> &th, bool on, i
     if (on) {
         if (G == 1 || th.d == 0) fx_line_at<N, EO, false, 0>(X + th.line(0), R + th.line(0), D);
         if (G == 1 || th.d == 1) fx_line_at<N, EO, false, 1>(X + th.line(1), S + th.line(1), D);
-        if (G == 3 && th.d == 2) fx_line_at<N, EO, false, 2>(X + th.line(2), TT + th.line(2), D);
+        if (G == 3 && th.d == 2) {
+            int m = 0;                 // the magnitudes' bits
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                const int h = X[th.line(2) + k * L].x;
+                m |= h ^ (h >> 31);
+            }
+            fx_line_at<N, EO, false, 2>(X + th.line(2), TT + th.line(2), D);
+            if (m != 0 && m < 1 << (30 - fx_grade(N))) *s_low = ~0u;
+        }
         if (th.has(0)) load(0, gb[0]);     // n = 2 with G = 3: the third thread owns no point
         if (K > 1 && th.has(1)) load(1, gb[1]);
     }
@@ -365,13 +382,24 @@ __device__ __forceinline__ fx::Pair fx_sum(const int2 *R, const int2 *S, const i
 // The largest biased exponent of an element's input: every thread's maximum of
 // the magnitudes' top words goes into the element's word of s_max (which is 0
 // before); the caller synchronises, then reads it with fx_emax.
+// The element's second word, s_max[EPC + el], says whether a column is small
+// (fx_note).  G = 1: it holds the smallest of the columns' maxima, zeros left
+// out, complemented; with one element per CTA it comes from the warps here, with
+// several from the threads that find theirs small once the element's is known
+// (fx_mark_small: a second atomic or warp reduction per element cost a CG iteration
+// 2 to 4 % at n = 4, 6 and 9, a register across the barrier 1 to 2 % at n = 10).
+// G = 3: the threads of the t lines mark it (fx_operator).
 template <int N, int G>
 __device__ __forceinline__ void fx_max_in(const FxThread<N, G> &th, bool on, unsigned top, unsigned *s_max) {
     constexpr int EPC = fx_epc(N, G);
     top = on ? top : 0u;
     if constexpr (EPC == 1) {
-        top = __reduce_max_sync(0xffffffffu, top);
-        if ((threadIdx.x & 31) == 0) atomicMax(s_max, top);
+        const unsigned a = __reduce_max_sync(0xffffffffu, top);
+        const unsigned l = G == 1 ? __reduce_max_sync(0xffffffffu, top ? ~top : 0u) : 0u;
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(s_max, a);
+            if (G == 1) atomicMax(s_max + 1, l);
+        }
     } else if constexpr (N >= 6) {      // a warp's threads belong to at most two elements
         const int first = (int)(threadIdx.x & ~31u) / (N * N);
         const unsigned a = __reduce_max_sync(0xffffffffu, th.el == first ? top : 0u);
@@ -457,6 +485,13 @@ __device__ __forceinline__ bool fx_on_face(unsigned cf, unsigned bf, int k) {
     return cf || (k == 0 && (bf & 16u)) || (k == N - 1 && (bf & 32u));
 }
 
+// The points k of the thread's column that are not on a face of the box, as bits.
+template <int N, int G>
+__device__ __forceinline__ unsigned fx_inner_points(const FxThread<N, G> &th, unsigned bf) {
+    const unsigned all = (1u << N) - 1u;
+    return (fx_column_faces(th) & bf) ? 0u : all & ~((bf >> 4) & 1u) & ~(((bf >> 5) & 1u) << (N - 1));
+}
+
 // The final pass of a CG head on a thread's points: w = the sum of the
 // partials in FP64, box faces zeroed; the points' products w p of the
 // fixed-point pairs, summed exactly over at most four points, go to
@@ -490,9 +525,236 @@ __device__ __forceinline__ void fx_final(const FxThread<N, G> &th, const int2 *X
         }
         flush(dA, dB);
     }
-    if (out.ext)
+    if (out.rest != 0) {
+        const double post = out.post();
+#pragma unroll 1
         for (int k = 0; k < K; k++)
-            if (th.has(k)) w[th.point(k) * N2] *= out.post;
+            if (th.has(k)) w[th.point(k) * N2] *= post;
+    }
+}
+
+// Graded elements.  A pair holds 54 bits below the element's largest entry, a
+// floating-point value the same number below its own.  So a point all of whose
+// inputs lie far below that entry loses as many bits here, and an element that
+// has such a point is computed again in double-float arithmetic (fx_redo_list),
+// which keeps 47 bits of every value.  The inputs of a point are above all those
+// on the three lines through it (the operator's leading terms).  A line is small
+// if its entries' exponents are all 8 or more below the element's largest (below
+// 2^-8 to 2^-7 of it; more at n = 2 and 3, whose lines have too few entries to
+// tell, fx_grade), and so is every line along a direction whose factors are below
+// 2^-6 of the element's largest.  An element is graded if all three lines of some
+// point are small, leaving out lines of zeros along t (on a face of the box,
+// where a field vanishes) and points on the box's faces, which the CG heads
+// zero; or if all its entries are tiny (kMinExp), or its word says so.
+// Why 8: on elements stretched by factors up to 100 and nine kinds of data
+// (emulated, n = 2 to 16) the largest error of a kept element is mostly below the
+// double-float operator's and at most 14 times as large (a single entry 2^7
+// above the others); without the rule it is up to 250 times.  And among 50000
+// elements of the directions of CG solves no column was small (n = 4 to 10).
+// A CTA lists elements that may be graded on the way (fx_note) and looks at them
+// again when it has done its share: with the test and the call inside the loop
+// over the elements the loop itself ran 2 to 5 % slower.  A graded element costs
+// three times another: 4096 of them at n = 10 take 262 us, others 80; in
+// double-float arithmetic alone they all took 119.
+// An element's word (ge): its exponent in the low 16 bits; kFxGraded: always
+// computed again (fx_factors_kernel); then one bit per direction with small
+// factors.
+constexpr int kFxExp = 0xffff, kFxGraded = 1 << 16, kFxWeak = 1 << 17;
+// The bits that put an element on the list whatever its input.
+constexpr int kFxSpecial = kFxGraded | (kFxWeak << 2);
+// The shift s of a point's factors (Scales) reaches about 2.4 log2(n) on a regular
+// element; an element where it is 5 more is graded.
+__host__ __device__ constexpr int fx_max_shift(int n) {
+    return 5 + (n < 3 ? 2 : (n < 4 ? 3 : (n < 6 ? 4 : (n < 8 ? 6 : (n < 10 ? 7 : (n < 13 ? 8 : 9))))));
+}
+
+// The factors of the elements, whole arrays, and what graded elements need.
+struct FxData {
+    const int4 *g;      // pairs [E][3][n^3], two per entry
+    const int *ge;      // the elements' words [E]
+    const double *gd;   // gxyz [E][6][n^3]
+    const void *dd;     // D in double-float pairs (DfConsts<N, EO>)
+    int gexp;           // biased exponent of max|gxyz|
+    int special;        // some element's word has one of kFxSpecial's bits
+    int2 *list;         // scratch [E]: the lists (fx_list)
+};
+
+// Puts an element on the CTA's list, by one thread.  The lists are chains through
+// the scratch: an entry holds the element before (-1: none) and the exponent of
+// the input; s_head: the last one listed.
+static __device__ __noinline__ void fx_list(const FxData &fd, int64_t e, int64_t end, unsigned top, int *s_head) {
+    if (e < end && top != 0u) fd.list[e] = make_int2(atomicExch(s_head, (int)e), (int)(top >> 20));
+}
+// With several elements in a CTA, or G = 3: a thread whose column is small marks
+// its element (fx_max_in).  With G = 3 it knows a third of the column only and
+// marks what the t lines do not see, entries whose integer is 0.
+template <int N, int G>
+__device__ __forceinline__ void fx_mark_small(const FxThread<N, G> &th, const FxData &fd, bool on, unsigned top,
+                                              unsigned elem, unsigned *s_max) {
+    if (on && top && (top + (unsigned)((G == 1 ? fx_grade(N) : 30) << 20) <= elem || elem < kFxTiny || fd.special))
+        s_max[fx_epc(N, G) + th.el] = ~0u;
+}
+// The list's upkeep, by the thread of each element of the CTA's group (e0, element
+// threadIdx.x): top is the element's first word of s_max, s_low the second ones,
+// which it clears.  The comparisons are all that an element costs that is not listed.
+template <int N, int G>
+__device__ __forceinline__ void fx_note(const FxData &fd, int64_t e0, int64_t end, unsigned top, unsigned *s_low,
+                                        int *s_head) {
+    const unsigned low = s_low[threadIdx.x];
+    bool may;
+    if (fx_epc(N, G) > 1 || G == 3) {
+        may = low != 0u;
+        if (may) s_low[threadIdx.x] = 0;
+    } else {
+        s_low[threadIdx.x] = 0;
+        may = low >= ~(top - (unsigned)(fx_grade(N) << 20)) || top < kFxTiny || fd.special;
+    }
+    if (may) fx_list(fd, e0 + threadIdx.x, end, top, s_head);
+}
+
+// One line of a graded element, one copy of its code: inlined, the lines would
+// share the entries of D they load, in spilled registers.
+template <int N, bool EO>
+__device__ __noinline__ void fx_redo_line(const float2 *in, float2 *out, int base, int stride,
+                                          const typename DfConsts<N, EO>::type *__restrict__ D, bool tr) {
+    if constexpr (EO) line_eo<N>(in, out, base, stride, tr ? D->bwd : D->fwd);
+    else line_plain<N>(in, out, base, stride, tr ? D->bwd : D->fwd);
+}
+
+// The lines through the points of a thread's column: are those along all three
+// directions small at one of the `points` (bits)?  X: the element's input in float
+// pairs, its largest entry in [1, 2).  weak: bits of directions whose lines all are.
+template <int N, int G>
+__device__ __forceinline__ bool fx_small_lines(const FxThread<N, G> &th, const float2 *X, int weak, unsigned points) {
+    constexpr int L = fx_layer(N);
+    auto small = [&](int dir, int at, int stride, bool zero_too) {
+        if ((weak >> dir) & 1) return true;
+        bool zero = true;
+#pragma unroll 1
+        for (int l = 0; l < N; l++) {
+            const float h = fabsf(X[at + l * stride].x);
+            if (h >= 2.f / (1 << fx_grade(N))) return false;
+            zero = zero && h == 0.f;
+        }
+        return zero_too || !zero;
+    };
+    if (!small(2, th.column(), L, false)) return false;
+#pragma unroll 1
+    for (int k = 0; k < N; k++)
+        if (((points >> k) & 1u) && small(0, N * th.j + L * k, 1, true) && small(1, th.i + L * k, N, true)) return true;
+    return false;
+}
+
+// A CTA's list, when it has done its share: w = ax_e(v) in double-float arithmetic
+// on those listed elements that are graded, zero on the box's faces if `mask`.
+// The layout and the phases are fx_operator's, the line products and scales
+// (an element's largest exponent, max|gxyz|) the double-float head's.  The sums
+// <w,p>_c keep the fixed-point products, whose error the large entries set.
+// Every thread calls it; sm holds the CTA's arrays, arrays of them per element.
+template <int N, bool EO, int G>
+__device__ __noinline__ void fx_redo_list(const FxData &fd, int head, const double *v, double *w, bool mask,
+                                          const Mesh &m, int2 *sm, int arrays) {
+    constexpr int N2 = N * N, N3 = N * N * N, A = fx_array(N), L = fx_layer(N), K = FxThread<N, G>::K;
+    constexpr int EPC = fx_epc(N, G);
+    __shared__ int2 s_slot[EPC];       // the elements at work and their exponents
+    __shared__ int s_next;
+    __shared__ unsigned s_graded;
+    FxThread<N, G> th;
+    th.init();
+    const auto *D = (const typename DfConsts<N, EO>::type *)fd.dd;
+    float2 *X = (float2 *)sm + arrays * A * th.el, *R = X + A, *S = X + 2 * A, *TT = arrays == 4 ? X + 3 * A : X;
+    const int at = th.column();
+    auto line = [&](const float2 *in, float2 *out, int dir, bool tr) {
+        fx_redo_line<N, EO>(in, out, th.line(dir), dir == 0 ? 1 : (dir == 1 ? N : L), D, tr);
+    };
+    for (; head >= 0; head = s_next) {
+        __syncthreads();               // the arrays and the shared words are free
+        if (threadIdx.x == 0) {
+            int e = head;
+            for (int el = 0; el < EPC; el++) {
+                s_slot[el] = make_int2(e, 0);
+                if (e < 0) continue;
+                const int2 entry = fd.list[e];
+                s_slot[el].y = entry.y;
+                e = entry.x;
+            }
+            s_next = e;
+            s_graded = 0;
+        }
+        __syncthreads();
+        const int64_t e = s_slot[th.el].x;
+        const int emax = s_slot[th.el].y;
+        const int word = e >= 0 ? fd.ge[e] : 0;
+        const int64_t q0 = e * N3 + at;
+        // not finite: the results are NaN already
+        bool on = th.active && e >= 0 && emax != 0x7ff && !(word & fx::kNotFinite);
+        unsigned bf = 0;
+        if (mask && on) {
+            int ex, ey, ez;
+            element_coords(e, m, ex, ey, ez);
+            bf = box_faces(ex, ey, ez, m);
+        }
+        if (on) {
+            double x[K];
+#pragma unroll
+            for (int kk = 0; kk < K; kk++)
+                if (th.has(kk)) x[kk] = v[q0 + th.point(kk) * N2];
+#pragma unroll
+            for (int kk = 0; kk < K; kk++)
+                if (th.has(kk)) X[at + th.point(kk) * L] = dfa::split_scaled(x[kk], 1023 - emax);
+        }
+        __syncthreads();
+        if (on && ((word & kFxGraded) || emax <= fx::kMinExp ||
+                   fx_small_lines(th, X, word / kFxWeak, fx_inner_points(th, bf))))
+            atomicOr(&s_graded, 1u << th.el);
+        __syncthreads();
+        on = on && ((s_graded >> th.el) & 1u);
+        if (on) {
+            if (G == 1 || th.d == 0) line(X, R, 0, false);
+            if (G == 1 || th.d == 1) line(X, S, 1, false);
+            if (G == 3 && th.d == 2) line(X, TT, 2, false);
+        }
+        __syncthreads();
+        if (on) {
+            if (G == 1) line(X, TT, 2, false);
+            const double *g = fd.gd + e * 6 * N3 + at;
+            double gv[2][6];            // a point's factors are loaded while the one before is contracted
+            auto load = [&](int kk) {
+#pragma unroll
+                for (int c = 0; c < 6; c++) gv[kk & 1][c] = g[(int64_t)c * N3 + th.point(kk) * N2];
+            };
+            if (th.has(0)) load(0);
+#pragma unroll 2
+            for (int kk = 0; kk < K; kk++) {
+                if (!th.has(kk)) break;
+                if (kk + 1 < K && th.has(kk + 1)) load(kk + 1);
+                const int q = at + th.point(kk) * L;
+                float2 f[6];
+#pragma unroll
+                for (int c = 0; c < 6; c++) f[c] = dfa::split_near(gv[kk & 1][c], 1023 - fd.gexp);
+                df_contract(f, R[q], S[q], TT[q]);
+            }
+            if (G == 1) line(TT, TT, 2, true);
+        }
+        __syncthreads();
+        if (on) {
+            if (G == 1 || th.d == 0) line(R, R, 0, true);
+            if (G == 1 || th.d == 1) line(S, S, 1, true);
+            if (G == 3 && th.d == 2) line(TT, TT, 2, true);
+        }
+        __syncthreads();
+        if (on) {
+            const unsigned cf = fx_column_faces(th) & bf;
+#pragma unroll 1
+            for (int kk = 0; kk < K; kk++) {
+                if (!th.has(kk)) break;
+                const int k = th.point(kk), q = at + k * L;
+                const double wv = dfa::join_scaled(dfa::add(dfa::add(R[q], S[q]), TT[q]),
+                                                   (emax - 1023) + (fd.gexp - 1023));
+                w[q0 + k * N2] = fx_on_face<N>(cf, bf, k) ? 0.0 : wv;
+            }
+        }
+    }
 }
 
 // Arguments of fx_elements (whole arrays).
@@ -503,24 +765,22 @@ struct FxIO {
     double *x;          // MODE 1: iterate (owed update applied when xa != 0)
     const double *minv; // MODE 1: Jacobi inverse diagonal (z = minv r), or null
     double *w;          // output
-    const int4 *g;      // factors [E][3][n^3], two per entry
-    const int *ge;      // their exponents [E], or null: ge0 for all
-    int ge0;
 };
 
 // ax_e on the elements e0 .. e0 + fx_epc(N, G) - 1 below e1, by the whole CTA
 // (every thread must call it; it contains barriers).  sm holds the arrays
-// without `keep`, s_max one word per element, 0 on entry and exit.  MODE 1 is
+// without `keep`, s_max two words per element, 0 on entry and exit.  MODE 1 is
 // the CG head of the forms that have their own kernels for the rest (Jacobi,
 // mask array): x += xa p, p = z + beta p, w = ax_e(p); with fuse, box-face
 // points of w are zeroed and the local products w p (p is continuous, so
 // their sum over all points is the assembled product) are added to dot.
 template <int N, int MODE, bool EO, int G>
-__device__ __forceinline__ void fx_elements(const FxIO &io, int64_t e0, int64_t e1, double beta, double xa, bool fuse,
-                                            const Mesh &m, const FxThread<N, G> &th,
+__device__ __forceinline__ void fx_elements(const FxIO &io, const FxData &fd, int64_t e0, int64_t e1, double beta,
+                                            double xa, bool fuse, const Mesh &m, const FxThread<N, G> &th,
                                             const typename FxConsts<N, EO>::type &D, int2 *sm, unsigned *s_max,
-                                            double &dot) {
+                                            int *s_head, double &dot) {
     constexpr int N2 = N * N, N3 = N * N * N, A = fx_array(N), L = fx_layer(N), K = FxThread<N, G>::K;
+    constexpr int EPC = fx_epc(N, G);
     const int64_t e = e0 + th.el;
     const bool on = th.active && e < e1;
     int2 *X = sm + 3 * A * th.el, *R = X + A, *S = X + 2 * A, *TT = G == 3 ? X + 3 * A : X;
@@ -542,15 +802,25 @@ __device__ __forceinline__ void fx_elements(const FxIO &io, int64_t e0, int64_t 
     }
     fx_max_in(th, on, top, s_max);
     __syncthreads();
-    const int emax = fx_emax(s_max[th.el]);
+    const unsigned elem = s_max[th.el];
+    const int emax = fx_emax(elem);
+    if (EPC > 1 || G == 3) fx_mark_small(th, fd, on, top, elem, s_max);
     if (on) fx_put_input(th, v, emax, X);
     __syncthreads();
-    if (threadIdx.x < fx_epc(N, G)) s_max[threadIdx.x] = 0;
-    fx_operator<N, EO>(th, on, X, R, S, TT, io.g + e * 3 * N3 + th.column(), D);
+    unsigned etop = 0;
+    if (threadIdx.x < EPC) {
+        etop = s_max[threadIdx.x];
+        s_max[threadIdx.x] = 0;
+    }
+    // loaded here: after the operator its latency showed (504 elements at n = 16
+    // 52.4 us instead of 51.3)
+    const int ge = on ? fd.ge[e] & kFxExp : 0;
+    fx_operator<N, EO>(th, on, X, R, S, TT, fd.g + e * 3 * N3 + th.column(), D, s_max + EPC);
+    if (threadIdx.x < EPC) fx_note<N, G>(fd, e0, e1, etop, s_max + EPC, s_head);
     __syncthreads();
     if (on) {
         fx::Scale out;
-        out.set(emax + (io.ge ? io.ge[e] : io.ge0) + D.so0);
+        out.set(emax + ge + D.so0);
         unsigned bf = 0;
         if (MODE == 1 && fuse) {
             int ex, ey, ez;
@@ -565,9 +835,12 @@ __device__ __forceinline__ void fx_elements(const FxIO &io, int64_t e0, int64_t 
             const double wv = out(fx_sum(R, S, TT, at + k * L));
             io.w[q0 + k * N2] = MODE == 1 && fuse && fx_on_face<N>(cf, bf, k) ? 0.0 : wv;
         }
-        if (out.ext)
+        if (out.rest != 0) {
+            const double post = out.post();
+#pragma unroll 1
             for (int kk = 0; kk < K; kk++)
-                if (th.has(kk)) io.w[q0 + th.point(kk) * N2] *= out.post;
+                if (th.has(kk)) io.w[q0 + th.point(kk) * N2] *= post;
+        }
         if (MODE == 1 && fuse) {
 #pragma unroll 4
             for (int kk = 0; kk < K; kk++) {
@@ -662,6 +935,16 @@ __device__ __forceinline__ int fx_point_exponent(const double (&v)[6], int (&ex)
     return e0 + (r > 0x7ffffffcull) + (r > 0xfffffff8ull);
 }
 
+// The directions of an element whose factors are small everywhere: gd holds the
+// largest biased exponents of its rr, ss and tt factors (the largest factor of a
+// positive definite matrix is one of them).
+__device__ __forceinline__ int fx_weak_bits(const int (&gd)[3]) {
+    const int top = gd[0] > gd[1] ? (gd[0] > gd[2] ? gd[0] : gd[2]) : (gd[1] > gd[2] ? gd[1] : gd[2]);
+    int bits = 0;
+    for (int d = 0; d < 3; d++) bits |= gd[d] < top - 6 ? kFxWeak << d : 0;
+    return bits;
+}
+
 // A point's factors with the row scales of D.
 __device__ __forceinline__ void fx_scale_point(double (&v)[6], int q, int n, const FxRows &rows) {
     const double a = rows.rho[q % n], b = rows.rho[(q / n) % n], c = rows.rho[q / (n * n)];
@@ -699,6 +982,27 @@ __device__ __forceinline__ void fx_point_pairs(const double (&v)[6], const int (
 #pragma unroll
     for (int c = 0; c < 3; c++) o[c] = make_int4(p[2 * c].x, p[2 * c].y, p[2 * c + 1].x, p[2 * c + 1].y);
 }
+
+// Does D lose precision in one scale?  Its pairs hold 55 bits below the largest
+// absolute row sum; a row or a column all of whose entries lie more than 2^7
+// below the largest entry keeps fewer than double-float pairs do.
+inline bool fx_graded_matrix(const double *D, int n) {
+    const FxScales S = fx_scales(D, n);
+    double top = 0.0, row[kMaxN] = {}, col[kMaxN] = {};
+    for (int i = 0; i < n; i++)
+        for (int l = 0; l < n; l++) {
+            const double v = fabs(D[i * n + l] * S.c[i]);
+            row[i] = fmax(row[i], v);
+            col[l] = fmax(col[l], v);
+            top = fmax(top, v);
+        }
+    for (int i = 0; i < n; i++)
+        if ((row[i] > 0.0 && row[i] < 0x1p-7 * top) || (col[i] > 0.0 && col[i] < 0x1p-7 * top)) return true;
+    return false;
+}
+
+// Floats of D's double-float tables in either form (DfConsts).
+constexpr int fx_df_floats(int n) { return 4 * n * n + 8 * (n + 1); }
 
 // v k to entry q: the product's rounding error goes to l.
 template <int M>

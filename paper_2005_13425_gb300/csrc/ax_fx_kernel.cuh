@@ -39,8 +39,7 @@ struct AxFxArgs {
     int finite;           // MODE 2: the operator's data (D and gxyz) has no NaN or Inf
     int fuse;             // MODE 1: zero box-face points, local products w p
     Mesh m;
-    const int4 *g;        // gxyz pairs [E][3][n^3], two per entry
-    const int *ge;        // their exponents [E]
+    FxData fd;
     int64_t E;
 };
 
@@ -84,7 +83,7 @@ __device__ __forceinline__ u128 fixed_of(long long v, int k, int lim, bool &out_
 template <int N, bool EO, int G>
 __device__ __forceinline__ u128 cg_head_pipelined(const AxFxArgs &a, double beta, double xa, int S128,
                                                   const typename FxConsts<N, EO>::type &D, int2 *sm,
-                                                  unsigned *s_max, bool &out_of_range) {
+                                                  unsigned *s_max, int *s_head, bool &out_of_range) {
     constexpr int N3 = N * N * N, A = fx_array(N), EPC = fx_epc(N, G);
     constexpr bool KEEP = fx_keep(N, G);
     __shared__ long long s_next;
@@ -93,10 +92,10 @@ __device__ __forceinline__ u128 cg_head_pipelined(const AxFxArgs &a, double beta
     int2 *X = sm + (KEEP ? 4 : 3) * A * th.el, *R = X + A, *S = X + 2 * A, *TT = KEEP ? X + 3 * A : X;
     const int col = th.column();
     double v[FxThread<N, G>::K];
+    unsigned top = 0;
     auto load = [&](int64_t e0) {   // the direction, kept in v
         const int64_t e = e0 + th.el, q = e * N3 + col;
         const bool on = th.active && e < a.E;
-        unsigned top = 0;
         if (on) {
             fx_direction<N, false>(th, a.r + q, a.p + q, a.x + q, nullptr, beta, xa, v);
             top = fx_top_of(th, v);
@@ -112,17 +111,23 @@ __device__ __forceinline__ u128 cg_head_pipelined(const AxFxArgs &a, double beta
         const bool on = th.active && e < a.E;
         unsigned nxt = 0;
         if (threadIdx.x == 0) nxt = atomicAdd(&a.sc->next_elem, 1u);
-        const int emax = fx_emax(s_max[th.el]);
+        const unsigned elem = s_max[th.el];
+        const int emax = fx_emax(elem);
+        if (EPC > 1) fx_mark_small(th, a.fd, on, top, elem, s_max);
         if (on) fx_put_input(th, v, emax, X);
         __syncthreads();
-        if (threadIdx.x < EPC) s_max[threadIdx.x] = 0;
-        fx_operator<N, EO>(th, on, X, R, S, TT, a.g + e * 3 * N3 + col, D);
+        if (threadIdx.x < EPC) {
+            const unsigned etop = s_max[threadIdx.x];
+            s_max[threadIdx.x] = 0;
+            fx_note<N, G>(a.fd, e0, a.E, etop, s_max + EPC, s_head);
+        }
+        fx_operator<N, EO>(th, on, X, R, S, TT, a.fd.g + e * 3 * N3 + col, D, s_max + EPC);
         if (threadIdx.x == 0) s_next = ((long long)gridDim.x + (long long)nxt) * EPC;
         __syncthreads();
         if (on) {   // w, and this thread's share of <w,p>_c into its exact sum
             int ex, ey, ez;
             element_coords(e, a.m, ex, ey, ez);
-            const int so = emax + a.ge[e] + D.so0;
+            const int so = emax + (a.fd.ge[e] & kFxExp) + D.so0;
             fx_final(th, X, R, S, TT, a.w + e * N3 + col, a.p + e * N3 + col, so, emax, box_faces(ex, ey, ez, a.m),
                      [&](long long dA, float dB) {
                          acc += fixed_of(dA + __float2ll_rn(dB), S128 + so + emax - 1052, a.dot_lim, out_of_range);
@@ -141,10 +146,11 @@ __device__ __forceinline__ u128 cg_head_pipelined(const AxFxArgs &a, double beta
 // registers and shared memory hold (fx_min_blocks).
 template <int N, int MODE, bool EO, int G>
 __global__ void __launch_bounds__(fx_threads(N, G), fx_min_blocks<N, G, MODE == 2 && fx_keep(N, G)>())
-ax_fx_kernel(AxFxArgs a, const __grid_constant__ typename FxConsts<N, EO>::type D) {
+ax_fx_kernel(const __grid_constant__ AxFxArgs a, const __grid_constant__ typename FxConsts<N, EO>::type D) {
     constexpr int EPC = fx_epc(N, G);
     extern __shared__ __align__(16) int2 sm[];
-    __shared__ unsigned s_max[EPC];
+    __shared__ unsigned s_max[2 * EPC];
+    __shared__ int s_head;      // of the list of elements that may be graded
     __shared__ double red[32];
     double beta = 0.0, xa = 0.0, dot = 0.0;
     if (MODE != 0) {
@@ -152,14 +158,16 @@ ax_fx_kernel(AxFxArgs a, const __grid_constant__ typename FxConsts<N, EO>::type 
         beta = a.sc->it == 0 ? 0.0 : a.sc->beta;
         xa = a.sc->x_alpha;
     }
-    if (threadIdx.x < EPC) s_max[threadIdx.x] = 0;
+    if (threadIdx.x < EPC) s_max[threadIdx.x] = s_max[EPC + threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_head = -1;
     __syncthreads();
     if constexpr (MODE == 2) {
         // the exact sums: per CTA, then over the CTAs by the last one
         const double pn = a.sc->it == 0 ? a.sc->rr : a.sc->pn2;
         const int S = a.dot_shift0 - ((int)((__double_as_longlong(pn) >> 52) & 0x7ff) - 1023);
         bool out_of_range = false;
-        const u128 mine = block_sum_u128(cg_head_pipelined<N, EO, G>(a, beta, xa, S, D, sm, s_max, out_of_range), red);
+        const u128 mine = block_sum_u128(cg_head_pipelined<N, EO, G>(a, beta, xa, S, D, sm, s_max, &s_head, out_of_range), red);
+        if (s_head >= 0) fx_redo_list<N, EO, G>(a.fd, s_head, a.p, a.w, true, a.m, sm, fx_keep(N, G) ? 4 : 3);
         finish_exact_sum(a.sc, a.partials, mine, S, out_of_range, a.finite && finite_pp(pn), red);
     } else {
         FxThread<N, G> th;
@@ -171,11 +179,12 @@ ax_fx_kernel(AxFxArgs a, const __grid_constant__ typename FxConsts<N, EO>::type 
         io.x = a.x;
         io.minv = a.minv;
         io.w = a.w;
-        io.g = a.g;
-        io.ge = a.ge;
-        io.ge0 = 0;
         for (int64_t e0 = (int64_t)blockIdx.x * EPC; e0 < a.E; e0 += (int64_t)gridDim.x * EPC)
-            fx_elements<N, MODE, EO, G>(io, e0, a.E, beta, xa, a.fuse != 0, a.m, th, D, sm, s_max, dot);
+            fx_elements<N, MODE, EO, G>(io, a.fd, e0, a.E, beta, xa, a.fuse != 0, a.m, th, D, sm, s_max,
+                                        &s_head, dot);
+        if (s_head >= 0)
+            fx_redo_list<N, EO, G>(a.fd, s_head, MODE == 0 ? a.u : a.p, a.w, MODE == 1 && a.fuse, a.m, sm,
+                                   G == 3 ? 4 : 3);
         if (MODE == 1 && a.fuse) {
             const double b = block_sum(dot, red);
             if (threadIdx.x == 0) a.partials[blockIdx.x] = b;
@@ -192,8 +201,8 @@ static nb_status launch_fx_nv(nb_ctx *c, const double *u, double *w, int mode) {
     int occ = 0;
     const auto &D = *reinterpret_cast<const typename FxConsts<N, EO>::type *>(c->fx_tab.data());
     AxFxArgs args{};
-    args.g = c->d_gxyz_fx;
-    args.ge = c->d_ge;
+    args.fd = {c->d_gxyz_fx, c->d_ge, c->d_gxyz, c->d_D_df, c->gxyz_exp, c->fx_special,
+               c->d_redo_list};
     args.E = c->m.E;
     if (mode == 0) {
         args.u = u;
@@ -244,9 +253,14 @@ void fx_tables_n(nb_ctx *c) {
         using T = std::remove_pointer_t<decltype(D)>;
         static_assert(sizeof(T) % sizeof(int4) == 0, "");
         c->fx_tab.resize(sizeof(T) / sizeof(int4));
+        constexpr bool EO = decltype(eo)::value;
+        using Df = typename DfConsts<N, EO>::type;
+        static_assert(sizeof(Df) <= sizeof(float) * fx_df_floats(N), "");
+        c->df_tab.resize(sizeof(Df) / sizeof(float));
         for (int q = 0; q < N * N; q++)
             if (!isfinite(c->D_host[q])) return;   // see prepare_fx
-        fx_consts<N, decltype(eo)::value>(c->D_host, *reinterpret_cast<T *>(c->fx_tab.data()));
+        fx_consts<N, EO>(c->D_host, *reinterpret_cast<T *>(c->fx_tab.data()));
+        df_consts<N, EO>(c->D_host, *reinterpret_cast<Df *>(c->df_tab.data()));
     };
     if (c->d_eo) make((typename FxConsts<N, true>::type *)nullptr, std::true_type{});
     else make((typename FxConsts<N, false>::type *)nullptr, std::false_type{});

@@ -160,6 +160,21 @@ __device__ __forceinline__ float2 split_scaled(double x, int sh) {
     return make_float2(h, l);
 }
 
+// The same with all 29 remaining bits in l, rounded to its 24 (|x 2^sh - (h + l)|
+// <= 2^-49 |x 2^sh|, the error of split); the scaled magnitude is below 2^128.
+__device__ __forceinline__ float2 split_near(double x, int sh) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned hi32 = (unsigned)(b >> 32), lo32 = (unsigned)b;
+    const int e = (int)((hi32 >> 20) & 0x7ffu), ef = e - 1023 + sh + 127;
+    if (e == 0 || ef < 1) return make_float2(0.f, 0.f);
+    const unsigned sign = hi32 & 0x80000000u;
+    const float h = __uint_as_float(sign | ((unsigned)ef << 23) | ((hi32 & 0xfffffu) << 3) | (lo32 >> 29));
+    float l = 0.f;
+    if (ef > 52)     // the unit of the 29 bits: 2^(ef - 127 - 52)
+        l = (float)(int)(lo32 & 0x1fffffffu) * __uint_as_float(sign | (unsigned)(ef - 52) << 23);
+    return make_float2(h, l);
+}
+
 // f * 2^so as a double, built with integer operations (f normal or zero).
 __device__ __forceinline__ double to_double_scaled(float f, int so) {
     const unsigned b = __float_as_uint(f);

@@ -140,22 +140,23 @@ __host__ __device__ __forceinline__ double scale2(double x, int k) {
 // rint(l 2^25) are doubles by construction (|l| < 64; worst case 33 for the
 // sum of the three partials at n = 16), and two FP64 FMAs scale them, add
 // them and take their offsets off: every step but the last is exact.
-// Outside +-900 (ext) the caller multiplies the results by a second factor,
+// Outside +-900 (rest) the caller multiplies the results by a second factor,
 // post, which brings the exponent to where it belongs (they then overflow or
 // underflow as FP64 does).  The same factor makes the results of an element with
 // non-finite data NaN.
 struct Scale {
-    double f, f2, c, post;
-    bool ext;
+    double f, f2, c;
+    int rest;            // what +-900 leaves of so
     __host__ __device__ __forceinline__ void set(int so) {
-        int s = so < -900 ? -900 : (so > 900 ? 900 : so);
+        const int s = so < -900 ? -900 : (so > 900 ? 900 : so);
         f = pow2(s);
         f2 = pow2(s - 25);
         c = -(4503599627370496.0 + 2147483648.0 + 134217728.0 + 64.0) * f;
-        ext = s != so;
-        s = so - s;
-        s = s < -1022 ? -1022 : (s > 1023 ? 1023 : s);
-        post = so > kNotFinite / 2 ? bits_d(0x7ff8000000000000ll) : pow2(s);
+        rest = so - s;
+    }
+    __host__ __device__ __forceinline__ double post() const {
+        if (rest > kNotFinite / 4) return bits_d(0x7ff8000000000000ll);
+        return pow2(rest < -1022 ? -1022 : (rest > 1023 ? 1023 : rest));
     }
     __host__ __device__ __forceinline__ double operator()(Pair p) const {
 #ifdef __CUDA_ARCH__

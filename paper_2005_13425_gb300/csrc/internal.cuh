@@ -118,8 +118,12 @@ struct nb_ctx {
     uint8_t *d_mask = nullptr;  // [E][n^3] or null (box mask)
     float *d_Df = nullptr;      // D as double-float pairs / fp32 (2*n*n)
     int4 *d_gxyz_fx = nullptr;  // [E][3][n^3] fixed-point pairs of gxyz, two per entry (ax_fx_core.cuh)
-    int *d_ge = nullptr;        // [E] their exponents (in d_gxyz_fx's allocation)
+    int *d_ge = nullptr;        // [E] the elements' words (ax_fx_core.cuh; in d_gxyz_fx's allocation)
+    float *d_D_df = nullptr;    // D in double-float pairs, for graded elements (DfConsts; in d_gxyz_fx's allocation)
     std::vector<int4> fx_tab;   // D's tables for that kernel (FxEo<n> or FxMat<n>)
+    std::vector<float> df_tab;  // what d_D_df holds
+    int2 *d_redo_list = nullptr;   // [E]: that kernel's lists of graded elements (in d_gxyz_fx's allocation)
+    int fx_special = 0;         // some element's word makes it suspect (ax_fx_core.cuh)
     int fx_dot_shift0 = 0, fx_dot_lim = 0;   // scale of the head's exact <w,p>_c (ax_fx.cu)
     float *d_gxyz32 = nullptr;  // [E][6][n^3] fp32 for the mixed inner solve
     float2 *d_gxyz_df = nullptr;  // [E][6][n^3] float pairs for the CG head on few elements (ax_df.cu; in d_gxyz_fx's allocation), or null

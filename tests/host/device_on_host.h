@@ -22,6 +22,8 @@ inline thread_local uint3 tid{0, 0, 0};
 inline uint3 bid{0, 0, 0};
 inline dim3 bdim(1), gdim(1);
 inline std::unique_ptr<std::barrier<>> bar;
+inline std::vector<std::unique_ptr<std::barrier<>>> wbar;   // one per warp
+inline std::vector<unsigned> lane;                          // a value per thread
 inline std::mutex mu;
 
 // Loads through __ldcs outside [lo, hi) are counted and answered with zeros.
@@ -32,6 +34,9 @@ inline long outside = 0;
 inline void cta(int threads, const std::function<void()> &body) {
     bdim = dim3(threads);
     bar = std::make_unique<std::barrier<>>(threads);
+    wbar.clear();
+    for (int w = 0; w < threads; w += 32) wbar.push_back(std::make_unique<std::barrier<>>(std::min(32, threads - w)));
+    lane.assign(threads, 0u);
     std::vector<std::thread> th;
     for (int t = 0; t < threads; t++)
         th.emplace_back([&, t] {
@@ -42,6 +47,10 @@ inline void cta(int threads, const std::function<void()> &body) {
 }
 }  // namespace host
 
+#undef __noinline__
+#define __noinline__
+#undef __shared__
+#define __shared__ static
 #define threadIdx (::host::tid)
 #define blockIdx (::host::bid)
 #define blockDim (::host::bdim)
@@ -104,16 +113,30 @@ inline T atomicMax(T *p, T v) {
     return o;
 }
 template <typename T>
+inline T atomicExch(T *p, T v) {
+    std::lock_guard<std::mutex> g(host::mu);
+    const T o = *p;
+    *p = v;
+    return o;
+}
+template <typename T>
 inline T atomicOr(T *p, T v) {
     std::lock_guard<std::mutex> g(host::mu);
     const T o = *p;
     *p = o | v;
     return o;
 }
-// The warp intrinsics are declared for the headers' other functions; nothing
-// here runs them, or gives a thread's own value where that is enough.
-inline unsigned __reduce_max_sync(unsigned, unsigned v) { return v; }
-inline int __reduce_max_sync(unsigned, int v) { return v; }
+inline unsigned __reduce_max_sync(unsigned, unsigned v) {   // all 32 lanes
+    const unsigned w = host::tid.x / 32, end = std::min<unsigned>(host::lane.size(), 32 * (w + 1));
+    host::lane[host::tid.x] = v;
+    host::wbar[w]->arrive_and_wait();
+    unsigned m = 0;
+    for (unsigned t = 32 * w; t < end; t++) m = std::max(m, host::lane[t]);
+    host::wbar[w]->arrive_and_wait();
+    return m;
+}
+inline int __reduce_max_sync(unsigned mask, int v) { return (int)__reduce_max_sync(mask, (unsigned)v); }   // v >= 0
+// Declared for the headers' other functions; nothing here calls it.
 template <typename T>
-inline T __shfl_down_sync(unsigned, T v, int) { return v; }
+T __shfl_down_sync(unsigned, T, int);
 inline void __threadfence() {}

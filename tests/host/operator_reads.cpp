@@ -16,6 +16,7 @@ static void run() {
     memset(D.get(), 0, sizeof *D);
     std::vector<int2> sm(4 * A);
     std::vector<int4> g(3 * N3);
+    unsigned low = 0;
     host::lo = (const char *)g.data();
     host::hi = (const char *)(g.data() + g.size());
     host::outside = 0;
@@ -24,7 +25,7 @@ static void run() {
         th.init();
         int2 *X = sm.data(), *R = X + A, *S = X + 2 * A, *TT = G == 3 ? X + 3 * A : X;
         const bool on = th.active && th.el == 0;    // one element; the CTA's others are past the end
-        fx_operator<N, EO>(th, on, X, R, S, TT, g.data() + th.column(), *D);
+        fx_operator<N, EO>(th, on, X, R, S, TT, g.data() + th.column(), *D, &low);
     });
     printf("%d %d %d %ld\n", N, (int)EO, G, host::outside);
 }
