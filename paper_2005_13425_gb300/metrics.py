@@ -124,9 +124,11 @@ def measured_peaks(root: str):
         return FALLBACK_HBM_GBS, FALLBACK_BF16_TFLOPS, "fallback"
 
 
-# Sources of the CG head kernel; a recorded DRAM traffic figure
+# Sources of the CG head kernel (all that it includes but internal.cuh, whose
+# device part is the mesh and the scalar block); a recorded DRAM traffic figure
 # is valid only for the sources it was measured on.
-CG_HEAD_SOURCES = ("ax_fx_kernel.cuh", "ax_fx_core.cuh", "fx.cuh", "reduce.cuh")
+CG_HEAD_SOURCES = ("ax_fx_kernel.cuh", "ax_fx_core.cuh", "ax_df_core.cuh", "df.cuh", "fx.cuh", "exact_sum.cuh",
+                   "reduce.cuh")
 
 
 _C_COMMENT = re.compile(r"//[^\n]*|/\*.*?\*/", re.S)
