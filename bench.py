@@ -599,12 +599,15 @@ def run_gpu(args, rank, world, local):
                 "avg_launch_ms": ax_avg_ms, "launches": ax["launches_timed"]}
     if fixed_point:
         # the fixed-point ax_e runs on the integer and FP32 pipes: its ALU bound
-        # is the instruction rate, its work the algorithm's multiply-adds
+        # is the rate of its terms (a wide multiply-add and two FFMA), its work the
+        # algorithm's multiply-adds
         ops = metrics.fx_instr_per_point(NGLL) * D
         ach = ops / (ax_avg_ms * 1e-3) / 1e12
-        roof_alu = {"bound": "alu", "achieved": ach, "peak": fp32_peak,
-                    "unit": "T instr/s", "frac": ach / fp32_peak, "traffic": traffic,
-                    "peak_source": "measured: nb_fp32_rate (FFMA rate, all SMs, this run); nominal "
+        fx_peak = metrics.fx_instr_rate(fp32_peak)
+        roof_alu = {"bound": "alu", "achieved": ach, "peak": fx_peak,
+                    "unit": "T instr/s", "frac": ach / fx_peak, "traffic": traffic,
+                    "peak_source": "measured: nb_fp32_rate (FFMA rate, all SMs, this run) x 3 x 33/121 (groups of a "
+                                   "wide multiply-add and two FFMA per FFMA); nominal FFMA rate "
                                    f"152 SMs x 128 lanes x 2070 MHz = {metrics.FP32_PEAK_TOPS:.2f}",
                     "kernel": "ax_e (CG head)", "algorithmic_instr_per_launch": ops,
                     "avg_launch_ms": ax_avg_ms, "launches": ax["launches_timed"]}

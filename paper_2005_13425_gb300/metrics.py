@@ -72,6 +72,18 @@ def fx_instr_per_point(n: int) -> float:
     return 3 * (6 * terms / n + 9)
 
 
+# A term's group of instructions against the FFMA rate: measured per SM and
+# clock, 121 FFMA, or 33 groups of one 32 x 32 + 64-bit multiply-add and two
+# FFMA (the wide multiply-add alone issues about 50 times).
+FX_GROUPS_PER_FFMA = 33.0 / 121.0
+
+
+def fx_instr_rate(ffma_rate: float) -> float:
+    """Instructions per second of the fixed-point terms (three per group) on a
+    device with this FFMA rate: the ceiling of fx_instr_per_point."""
+    return 3 * FX_GROUPS_PER_FFMA * ffma_rate
+
+
 def cg_flops_per_point(n: int) -> int:
     """Eq. 1: flops per degree of freedom per CG iteration."""
     return 12 * n + 34
