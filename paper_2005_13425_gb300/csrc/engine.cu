@@ -1430,7 +1430,8 @@ nb_status engine_submit_internal(nb_engine *g, nb_box box, int n, double amp, co
 }
 
 // The stream of branch k of a capture: the engine's own stream for the first
-// group, a side stream for each further one.
+// group, a side stream of the same priority for each further one (a captured
+// kernel keeps the priority of the stream it was captured on).
 static nb_status branch_stream(nb_engine *g, int k, cudaStream_t *out) {
     if (k == 0) {
         *out = g->stream;
@@ -1440,19 +1441,26 @@ static nb_status branch_stream(nb_engine *g, int k, cudaStream_t *out) {
     if (!g->join) NB_CUDA(cudaEventCreateWithFlags(&g->join, cudaEventDisableTiming));
     while ((int)g->branches.size() < k) {
         cudaStream_t st = nullptr;
-        NB_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+        int priority = 0;
+        NB_CUDA(cudaStreamGetPriority(g->stream, &priority));
+        NB_CUDA(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, priority));
         g->branches.push_back(st);
     }
     *out = g->branches[k - 1];
     return NB_OK;
 }
 
-// FP64 groups of more elements than this take turns in one branch: a group
-// that fills the GPU by itself loses more by sharing the L2 with another than
-// its tail costs.  100 iterations of
-// FP64 requests at n = 6 to 12, all in turn against all as branches: 232.7 and
-// 221 ms with 7 to 17 thousand elements per group, 309.7 and 305 with 18 to 23,
-// 476.9 and 481 with 22 to 38, 1148 and 1194 with 57 to 91.
+// FP64 groups of more elements than this take turns in one branch: of groups that
+// fill the GPU by themselves the branches gain less and less, and then lose.
+// 100 iterations of FP64 requests at n = 6 to 12, all in turn against all as
+// branches: 232.7 and 221 ms with 7 to 17 thousand elements per group, 309.7 and 305
+// with 18 to 23, 476.9 and 481 with 22 to 38, 1148 and 1194 with 57 to 91.  With the
+// limit no mix was found slower than in turn; one iteration, in turn and now:
+// 4096 elements at each of n = 13 to 16 4.28 and 3.72 ms, 16384 at n = 15 and 16 9.33
+// and 9.02, 18000 at n = 3 and 4 0.194 and 0.129, 32768 at n = 10 beside mixed groups of
+// 16384 at n = 8 and 12 2.26 and 2.00, 32768 at n = 3, 4 and 5 (above the limit) 0.52 both.
+// The element count does not see n: whether small orders gain as branches above
+// the limit was not measured.
 static int64_t branch_elements(const nb_engine *g) { return (int64_t)128 * g->sms; }
 
 // One engine step is a captured graph of `chunk` iterations with one branch per
