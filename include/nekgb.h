@@ -264,9 +264,14 @@ nb_status nb_jacobi_diagonal(nb_ctx *ctx, double *minv_dev);
 nb_status nb_solve_stats(const nb_ctx *ctx, int *iters, int *outer);
 
 /* Select the ax_e kernel: 0 = automatic (fastest FP64-accurate kernel),
- * 1 = native FP64 layer kernel, 2 = the kernel on the integer and FP32 pipes
- * (fixed-point pairs; the automatic choice at every n).  All variants meet
- * the same accuracy contract. */
+ * 1 = native FP64 layer kernel, 2 = the kernels on the integer and FP32 pipes
+ * (the automatic choice at every n): fixed-point pairs, and double-float pairs
+ * in the unpreconditioned CG on boxes of few elements and on elements whose
+ * data spans many orders of magnitude.  All variants meet the same accuracy
+ * contract: the error is relative to the largest result of an element (about
+ * 2^-50 of its terms); entries far below it are accurate to about 2^-47 of their
+ * own terms once these lie 2^8 below.  Variant 1 keeps FP64 accuracy for every
+ * entry.  A NaN or Inf in an element's input or factors makes its results NaN. */
 nb_status nb_set_ax_variant(nb_ctx *ctx, int variant);
 
 /* --------------------------------------------------------------------- */

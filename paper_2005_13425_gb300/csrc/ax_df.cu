@@ -2,9 +2,9 @@
 // pairs (df.cuh, ax_df_core.cuh): x += xa p, p = r + beta p, w = ax_e(p) and
 // <w,p>_c.  Such solves run past convergence within the paper's fixed 100
 // iterations, where CG amplifies the rounding of its operator to 1e-9 and more
-// of x; with the arithmetic kept, their results stay what they were.  On 64
-// elements at n = 8 an iteration takes 18.0 us with it and with the fixed-point
-// head (ax_fx_kernel.cuh); before its loads were batched it took 20.5.
+// of x; with the arithmetic kept, their results stay what they were (the
+// fixed-point operator is no less accurate).  On one CTA per SM and fewer it is
+// also the faster head for most orders (df_head_elements).
 //
 // Thread layout ("line threads").  A CTA owns one element at a time and has
 // 3 n^2 working threads: thread (d, a0, a1) owns one line of the element
@@ -253,7 +253,14 @@ __global__ void split_scaled_kernel(const double *__restrict__ x, float2 *__rest
 }
 
 // The boxes that take this head: those whose fixed-point head would have at
-// most two CTAs per SM (several elements each for n < 8 and n = 9).
+// most two CTAs per SM (several elements each for n < 8 and n = 9).  A CG iteration
+// with this head and with the fixed-point one, us, at 38, 152 and 304 CTAs' elements:
+//   n = 2   28.1/17.9  55.2/17.9  58.2/18.8      n = 10  19.6/23.4  20.4/26.0  26.1/26.3
+//   n = 4   16.5/16.8  24.0/20.6  29.9/21.9      n = 12  23.0/28.4  24.9/31.8  33.3/33.4
+//   n = 6   16.1/17.8  19.7/20.6  25.3/23.9      n = 14  34.2/34.3  36.4/37.9  63.5/43.6
+//   n = 8   17.1/20.8  17.7/22.8  20.3/22.1      n = 16  46.4/41.8  51.0/45.7  88.9/53.8
+// So by time alone the line would lie lower at n <= 4 and at n >= 13 (where this head
+// holds one CTA per SM); it lies here because the results of these boxes were kept.
 bool df_head_elements(int64_t E, int n) {
     const int epc = n == 8 || n >= 10 ? 1 : (n >= 6 ? 3 : 128 / (n * n));
     return (E + epc - 1) / epc <= (int64_t)2 * device_sms();

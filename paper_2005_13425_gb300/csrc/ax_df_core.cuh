@@ -1,7 +1,8 @@
 // Double-float ax_e (Listing 1, arXiv 2005.13425 Sec. III) on FP32 pairs
 // (df.cuh) for the batched engine (engine.cu), the CG head on boxes of few
-// elements (ax_df.cu) and the measurement probe (probe_tc.cu): derivative-matrix constants, the even-odd line product and
-// one element of the operator.
+// elements (ax_df.cu), the fixed-point kernels' graded elements
+// (ax_fx_core.cuh) and the measurement probe (probe_tc.cu): derivative-matrix
+// constants, the line products and one element of the operator.
 #pragma once
 
 #include "df.cuh"
@@ -94,8 +95,8 @@ __device__ __forceinline__ int line_of(int task, int &stride) {
 }
 
 // out(base + m*stride) = sum_l M(m,l) in(base + l*stride) in even-odd form
-// (see EoMat): pair sums and
-// differences, then 2 dot products of N/2 terms per output pair.
+// (see EoMat): pair sums and differences, then 2 dot products of N/2 terms per
+// output pair.
 template <int N>
 __device__ __forceinline__ void line_eo(const float2 *in, float2 *out, int base, int stride,
                                         const EoMat<N> &M) {

@@ -1,8 +1,8 @@
 // Core of the FP64-accurate ax_e (Listing 1, arXiv 2005.13425 Sec. III) in
-// fixed-point pairs (fx.cuh), shared by the single-problem kernel (ax_fx.cu)
-// and the batched engine (engine.cu): the scaled derivative-matrix constants,
-// the line products (plain and even-odd), the phases of one element and the
-// conversion of the geometric factors.
+// fixed-point pairs (fx.cuh) for the kernels of ax_fx_kernel.cuh: the scaled
+// derivative-matrix constants, the line products (plain and even-odd), the
+// phases of one element, the elements that are computed again in double-float
+// arithmetic, and the conversion of the geometric factors.
 //
 // Scales.
 //  * The rows of D are brought to similar size and the geometric factors take
