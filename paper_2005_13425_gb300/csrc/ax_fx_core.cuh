@@ -576,14 +576,35 @@ struct FxData {
     const void *dd;     // D in double-float pairs (DfConsts<N, EO>)
     int gexp;           // biased exponent of max|gxyz|
     int special;        // some element's word has one of kFxSpecial's bits
-    int2 *list;         // scratch [E]: the lists (fx_list)
+    int2 *list;         // scratch [E]: the CG heads' lists (FxList)
 };
 
-// Puts an element on the CTA's list, by one thread.  The lists are chains through
-// the scratch: an entry holds the element before (-1: none) and the exponent of
-// the input; s_head: the last one listed.
-static __device__ __noinline__ void fx_list(const FxData &fd, int64_t e, int64_t end, unsigned top, int *s_head) {
-    if (e < end && top != 0u) fd.list[e] = make_int2(atomicExch(s_head, (int)e), (int)(top >> 20));
+// A CTA's list of elements that may be graded.  CHAIN (the CG heads, whose CTAs
+// take many groups): a chain through the scratch, an entry holding the element
+// before (-1: none) and the exponent of the input; head: the last one listed.
+// Otherwise (MODE 0: one group per CTA) the group's own slots, (element or -1,
+// exponent), so that the operator alone keeps no state between or beside its launches;
+// head >= 0: there is one.
+template <int EPC, bool CHAIN>
+struct FxList {
+    int head;
+    int2 slot[CHAIN ? 1 : EPC];
+    __device__ __forceinline__ void init() {
+        if (threadIdx.x == 0) head = -1;
+        if (!CHAIN && threadIdx.x < EPC) slot[threadIdx.x].x = -1;
+    }
+};
+// Puts an element on it, by one thread.
+template <int EPC, bool CHAIN>
+__device__ __noinline__ void fx_list(const FxData &fd, int64_t e, int64_t end, unsigned top,
+                                     FxList<EPC, CHAIN> &list) {
+    if (e >= end || top == 0u) return;
+    if (CHAIN) {
+        fd.list[e] = make_int2(atomicExch(&list.head, (int)e), (int)(top >> 20));
+    } else {
+        list.slot[CHAIN ? 0 : threadIdx.x] = make_int2((int)e, (int)(top >> 20));
+        list.head = 0;
+    }
 }
 // With several elements in a CTA, or G = 3: a thread whose column is small marks
 // its element (fx_max_in).  With G = 3 it knows a third of the column only and
@@ -597,9 +618,9 @@ __device__ __forceinline__ void fx_mark_small(const FxThread<N, G> &th, const Fx
 // The list's upkeep, by the thread of each element of the CTA's group (e0, element
 // threadIdx.x): top is the element's first word of s_max, s_low the second ones,
 // which it clears.  The comparisons are all that an element costs that is not listed.
-template <int N, int G>
+template <int N, int G, bool CHAIN>
 __device__ __forceinline__ void fx_note(const FxData &fd, int64_t e0, int64_t end, unsigned top, unsigned *s_low,
-                                        int *s_head) {
+                                        FxList<fx_epc(N, G), CHAIN> &list) {
     const unsigned low = s_low[threadIdx.x];
     bool may;
     if (fx_epc(N, G) > 1 || G == 3) {
@@ -609,7 +630,7 @@ __device__ __forceinline__ void fx_note(const FxData &fd, int64_t e0, int64_t en
         s_low[threadIdx.x] = 0;
         may = low >= ~(top - (unsigned)(fx_grade(N) << 20)) || top < kFxTiny || fd.special;
     }
-    if (may) fx_list(fd, e0 + threadIdx.x, end, top, s_head);
+    if (may) fx_list(fd, e0 + threadIdx.x, end, top, list);
 }
 
 // One line of a graded element, one copy of its code: inlined, the lines would
@@ -651,9 +672,9 @@ __device__ __forceinline__ bool fx_small_lines(const FxThread<N, G> &th, const f
 // (an element's largest exponent, max|gxyz|) the double-float head's.  The sums
 // <w,p>_c keep the fixed-point products, whose error the large entries set.
 // Every thread calls it; sm holds the CTA's arrays, arrays of them per element.
-template <int N, bool EO, int G>
-__device__ __noinline__ void fx_redo_list(const FxData &fd, int head, const double *v, double *w, bool mask,
-                                          const Mesh &m, int2 *sm, int arrays) {
+template <int N, bool EO, int G, bool CHAIN>
+__device__ __noinline__ void fx_redo_list(const FxData &fd, const FxList<fx_epc(N, G), CHAIN> &list, const double *v,
+                                          double *w, bool mask, const Mesh &m, int2 *sm, int arrays) {
     constexpr int N2 = N * N, N3 = N * N * N, A = fx_array(N), L = fx_layer(N), K = FxThread<N, G>::K;
     constexpr int EPC = fx_epc(N, G);
     __shared__ int2 s_slot[EPC];       // the elements at work and their exponents
@@ -667,18 +688,24 @@ __device__ __noinline__ void fx_redo_list(const FxData &fd, int head, const doub
     auto line = [&](const float2 *in, float2 *out, int dir, bool tr) {
         fx_redo_line<N, EO>(in, out, th.line(dir), dir == 0 ? 1 : (dir == 1 ? N : L), D, tr);
     };
-    for (; head >= 0; head = s_next) {
+    int head = list.head;
+    // a chain has an element at most once; the bound ends the walk whatever it holds
+    for (int64_t left = m.E; head >= 0 && left > 0; head = s_next, left--) {
         __syncthreads();               // the arrays and the shared words are free
         if (threadIdx.x == 0) {
             int e = head;
             for (int el = 0; el < EPC; el++) {
+                if (!CHAIN) {
+                    s_slot[el] = list.slot[CHAIN ? 0 : el];
+                    continue;
+                }
                 s_slot[el] = make_int2(e, 0);
                 if (e < 0) continue;
                 const int2 entry = fd.list[e];
                 s_slot[el].y = entry.y;
                 e = entry.x;
             }
-            s_next = e;
+            s_next = CHAIN ? e : -1;
             s_graded = 0;
         }
         __syncthreads();
@@ -778,7 +805,7 @@ template <int N, int MODE, bool EO, int G>
 __device__ __forceinline__ void fx_elements(const FxIO &io, const FxData &fd, int64_t e0, int64_t e1, double beta,
                                             double xa, bool fuse, const Mesh &m, const FxThread<N, G> &th,
                                             const typename FxConsts<N, EO>::type &D, int2 *sm, unsigned *s_max,
-                                            int *s_head, double &dot) {
+                                            FxList<fx_epc(N, G), MODE != 0> &list, double &dot) {
     constexpr int N2 = N * N, N3 = N * N * N, A = fx_array(N), L = fx_layer(N), K = FxThread<N, G>::K;
     constexpr int EPC = fx_epc(N, G);
     const int64_t e = e0 + th.el;
@@ -816,7 +843,7 @@ __device__ __forceinline__ void fx_elements(const FxIO &io, const FxData &fd, in
     // 52.4 us instead of 51.3)
     const int ge = on ? fd.ge[e] & kFxExp : 0;
     fx_operator<N, EO>(th, on, X, R, S, TT, fd.g + e * 3 * N3 + th.column(), D, s_max + EPC);
-    if (threadIdx.x < EPC) fx_note<N, G>(fd, e0, e1, etop, s_max + EPC, s_head);
+    if (threadIdx.x < EPC) fx_note<N, G>(fd, e0, e1, etop, s_max + EPC, list);
     __syncthreads();
     if (on) {
         fx::Scale out;

@@ -83,7 +83,8 @@ __device__ __forceinline__ u128 fixed_of(long long v, int k, int lim, bool &out_
 template <int N, bool EO, int G>
 __device__ __forceinline__ u128 cg_head_pipelined(const AxFxArgs &a, double beta, double xa, int S128,
                                                   const typename FxConsts<N, EO>::type &D, int2 *sm,
-                                                  unsigned *s_max, int *s_head, bool &out_of_range) {
+                                                  unsigned *s_max, FxList<fx_epc(N, G), true> &list,
+                                                  bool &out_of_range) {
     constexpr int N3 = N * N * N, A = fx_array(N), EPC = fx_epc(N, G);
     constexpr bool KEEP = fx_keep(N, G);
     __shared__ long long s_next;
@@ -119,7 +120,7 @@ __device__ __forceinline__ u128 cg_head_pipelined(const AxFxArgs &a, double beta
         if (threadIdx.x < EPC) {
             const unsigned etop = s_max[threadIdx.x];
             s_max[threadIdx.x] = 0;
-            fx_note<N, G>(a.fd, e0, a.E, etop, s_max + EPC, s_head);
+            fx_note<N, G>(a.fd, e0, a.E, etop, s_max + EPC, list);
         }
         fx_operator<N, EO>(th, on, X, R, S, TT, a.fd.g + e * 3 * N3 + col, D, s_max + EPC);
         if (threadIdx.x == 0) s_next = ((long long)gridDim.x + (long long)nxt) * EPC;
@@ -150,7 +151,7 @@ ax_fx_kernel(const __grid_constant__ AxFxArgs a, const __grid_constant__ typenam
     constexpr int EPC = fx_epc(N, G);
     extern __shared__ __align__(16) int2 sm[];
     __shared__ unsigned s_max[2 * EPC];
-    __shared__ int s_head;      // of the list of elements that may be graded
+    __shared__ FxList<EPC, MODE != 0> list;
     __shared__ double red[32];
     double beta = 0.0, xa = 0.0, dot = 0.0;
     if (MODE != 0) {
@@ -159,15 +160,15 @@ ax_fx_kernel(const __grid_constant__ AxFxArgs a, const __grid_constant__ typenam
         xa = a.sc->x_alpha;
     }
     if (threadIdx.x < EPC) s_max[threadIdx.x] = s_max[EPC + threadIdx.x] = 0;
-    if (threadIdx.x == 0) s_head = -1;
+    list.init();
     __syncthreads();
     if constexpr (MODE == 2) {
         // the exact sums: per CTA, then over the CTAs by the last one
         const double pn = a.sc->it == 0 ? a.sc->rr : a.sc->pn2;
         const int S = a.dot_shift0 - ((int)((__double_as_longlong(pn) >> 52) & 0x7ff) - 1023);
         bool out_of_range = false;
-        const u128 mine = block_sum_u128(cg_head_pipelined<N, EO, G>(a, beta, xa, S, D, sm, s_max, &s_head, out_of_range), red);
-        if (s_head >= 0) fx_redo_list<N, EO, G>(a.fd, s_head, a.p, a.w, true, a.m, sm, fx_keep(N, G) ? 4 : 3);
+        const u128 mine = block_sum_u128(cg_head_pipelined<N, EO, G>(a, beta, xa, S, D, sm, s_max, list, out_of_range), red);
+        if (list.head >= 0) fx_redo_list<N, EO, G>(a.fd, list, a.p, a.w, true, a.m, sm, fx_keep(N, G) ? 4 : 3);
         finish_exact_sum(a.sc, a.partials, mine, S, out_of_range, a.finite && finite_pp(pn), red);
     } else {
         FxThread<N, G> th;
@@ -181,9 +182,9 @@ ax_fx_kernel(const __grid_constant__ AxFxArgs a, const __grid_constant__ typenam
         io.w = a.w;
         for (int64_t e0 = (int64_t)blockIdx.x * EPC; e0 < a.E; e0 += (int64_t)gridDim.x * EPC)
             fx_elements<N, MODE, EO, G>(io, a.fd, e0, a.E, beta, xa, a.fuse != 0, a.m, th, D, sm, s_max,
-                                        &s_head, dot);
-        if (s_head >= 0)
-            fx_redo_list<N, EO, G>(a.fd, s_head, MODE == 0 ? a.u : a.p, a.w, MODE == 1 && a.fuse, a.m, sm,
+                                        list, dot);
+        if (list.head >= 0)
+            fx_redo_list<N, EO, G>(a.fd, list, MODE == 0 ? a.u : a.p, a.w, MODE == 1 && a.fuse, a.m, sm,
                                    G == 3 ? 4 : 3);
         if (MODE == 1 && a.fuse) {
             const double b = block_sum(dot, red);
@@ -235,9 +236,9 @@ static nb_status launch_fx_nv(nb_ctx *c, const double *u, double *w, int mode) {
     const int64_t cap = (int64_t)device_sms() * occ, need = (c->m.E + EPC - 1) / EPC;
     // the operator alone: one CTA per group of elements, which the hardware
     // hands out as SMs become free (a resident grid striding over 4096 elements
-    // at n = 10 idled a tenth of the time in its last round); the heads: a
-    // resident grid, one reduction per CTA
-    const int64_t most = mode == 0 ? (int64_t)1 << 30 : cap;
+    // at n = 10 idled a tenth of the time in its last round; FxList relies on one
+    // group); the heads: a resident grid, one reduction per CTA
+    const int64_t most = mode == 0 ? (int64_t)0x7fffffff : cap;
     const int grid = (int)(need < most ? need : most);
     if (mode == 1) c->ax_grid = grid;
     LaunchTimer tm(c, NB_K_AX);

@@ -122,7 +122,7 @@ struct nb_ctx {
     float *d_D_df = nullptr;    // D in double-float pairs, for graded elements (DfConsts; in d_gxyz_fx's allocation)
     std::vector<int4> fx_tab;   // D's tables for that kernel (FxEo<n> or FxMat<n>)
     std::vector<float> df_tab;  // what d_D_df holds
-    int2 *d_redo_list = nullptr;   // [E]: that kernel's lists of graded elements (in d_gxyz_fx's allocation)
+    int2 *d_redo_list = nullptr;   // [E]: the CG heads' lists of graded elements (in d_gxyz_fx's allocation)
     int fx_special = 0;         // some element's word makes it suspect (ax_fx_core.cuh)
     int fx_dot_shift0 = 0, fx_dot_lim = 0;   // scale of the head's exact <w,p>_c (ax_fx.cu)
     float *d_gxyz32 = nullptr;  // [E][6][n^3] fp32 for the mixed inner solve

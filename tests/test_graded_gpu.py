@@ -103,6 +103,42 @@ def test_operator(nek, oracle, n, few, kind):
     assert err[1::2].max() <= (1e-12 if kind == "matrix" else 2e-14)
 
 
+@pytest.mark.parametrize("n,few", [(4, False), (8, True), (10, False)])
+def test_operator_beside_itself(nek, oracle, n, few):
+    """nb_ax keeps nothing between its launches: two captured calls of one context,
+    replayed on two streams at a time, give the bits they give alone."""
+    dims = boxes(n, few)
+    P = oracle.box_problem(*dims, n, inputs.PERTURB_AMP, inputs.perturbation_coeffs(n))
+    stream = torch.cuda.current_stream()
+    h = nek.nb_setup(dims, n, P["D"], P["gxyz"], stream=stream)
+    try:
+        us = [torch.from_numpy(graded(kind, P, n)[2]).cuda() for kind in ("spike", "corner")]
+        alone, outs, graphs = [], [], []
+        for u in us:
+            w = torch.empty_like(u)
+            nek.nb_ax(h, u, w)
+            stream.synchronize()
+            alone.append(w.clone())
+            outs.append(w)
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+                nek.nb_ax(h, u, w)
+            graphs.append(g)
+        sides = [torch.cuda.Stream(), torch.cuda.Stream()]
+        for w in outs:
+            w.fill_(7.0)
+        torch.cuda.synchronize()
+        for _ in range(20):
+            for g, side in zip(graphs, sides):
+                with torch.cuda.stream(side):
+                    g.replay()
+        torch.cuda.synchronize()
+        for w, want in zip(outs, alone):
+            assert torch.equal(w.view(torch.int64), want.view(torch.int64))
+    finally:
+        nek.nb_destroy(h)
+
+
 @pytest.mark.parametrize("jacobi", [False, True])
 @pytest.mark.parametrize("n,dims", [(8, (13, 7, 5)), (13, (11, 7, 5))])
 def test_cg_heads(nek, oracle, n, dims, jacobi):
