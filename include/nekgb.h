@@ -269,9 +269,10 @@ nb_status nb_solve_stats(const nb_ctx *ctx, int *iters, int *outer);
  * in the unpreconditioned CG on boxes of few elements and on elements whose
  * data spans many orders of magnitude.  All variants meet the same accuracy
  * contract: the error is relative to the largest result of an element (about
- * 2^-50 of its terms); entries far below it are accurate to about 2^-47 of their
- * own terms once these lie 2^8 below.  Variant 1 keeps FP64 accuracy for every
- * entry.  A NaN or Inf in an element's input or factors makes its results NaN. */
+ * 2^-50 of its terms); at points whose inputs along all three directions lie 2^8
+ * and more below the element's largest it is about 2^-47 of the point's own
+ * terms.  Variant 1 keeps FP64 accuracy for every entry.  A NaN or Inf in an
+ * element's input or factors makes its results NaN. */
 nb_status nb_set_ax_variant(nb_ctx *ctx, int variant);
 
 /* --------------------------------------------------------------------- */

@@ -142,7 +142,7 @@ __host__ __device__ constexpr int fx_min_blocks() {
 
 // Exponents below the element's largest from which entries count as small (see
 // Graded elements).
-__host__ __device__ constexpr int fx_grade(int n) { return n == 2 ? 11 : (n == 3 ? 10 : 8); }
+__host__ __device__ constexpr int fx_grade(int n) { return n <= 3 ? 10 : 8; }
 // Top words of elements that are graded because all their entries are tiny.
 constexpr unsigned kFxTiny = (unsigned)(fx::kMinExp + 1) << 20;
 
@@ -542,13 +542,15 @@ __device__ __forceinline__ void fx_final(const FxThread<N, G> &th, const int2 *X
 // if its entries' exponents are all 8 or more below the element's largest (below
 // 2^-8 to 2^-7 of it; more at n = 2 and 3, whose lines have too few entries to
 // tell, fx_grade), and so is every line along a direction whose factors are below
-// 2^-6 of the element's largest.  An element is graded if all three lines of some
+// 2^-14 of the element's largest (sides 128 : 1; with t such a direction all
+// elements are listed, and at 2^-6 flat boxes of 16 layers to one ran 11 to 18 %
+// slower).  An element is graded if all three lines of some
 // point are small, leaving out lines of zeros along t (on a face of the box,
 // where a field vanishes) and points on the box's faces, which the CG heads
 // zero; or if all its entries are tiny (kMinExp), or its word says so.
 // Why 8: on elements stretched by factors up to 100 and nine kinds of data
 // (emulated, n = 2 to 16) the largest error of a kept element is mostly below the
-// double-float operator's and at most 14 times as large (a single entry 2^7
+// double-float operator's and at most 18 times as large (a single entry 2^7
 // above the others); without the rule it is up to 250 times.  And among 50000
 // elements of the directions of CG solves no column was small (n = 4 to 10).
 // A CTA lists elements that may be graded on the way (fx_note) and looks at them
@@ -968,7 +970,7 @@ __device__ __forceinline__ int fx_point_exponent(const double (&v)[6], int (&ex)
 __device__ __forceinline__ int fx_weak_bits(const int (&gd)[3]) {
     const int top = gd[0] > gd[1] ? (gd[0] > gd[2] ? gd[0] : gd[2]) : (gd[1] > gd[2] ? gd[1] : gd[2]);
     int bits = 0;
-    for (int d = 0; d < 3; d++) bits |= gd[d] < top - 6 ? kFxWeak << d : 0;
+    for (int d = 0; d < 3; d++) bits |= gd[d] < top - 14 ? kFxWeak << d : 0;
     return bits;
 }
 

@@ -64,6 +64,9 @@ def graded(kind, P, n):
     elif kind == "tiny":                                         # the largest entry is below 2^-958
         u[even] *= 1e-295
         g *= 1e40                                                # w itself stays a normal number
+    elif kind == "flat":                                         # t sides 512 times as long: weak factors
+        u[even] *= np.repeat(2.0 ** (-30 * t), n * n)
+        g[even] *= np.array([512.0, 512.0, 1.0, 512.0, 1.0, 1.0 / 512.0])[:, None]
     elif kind == "jacobian":
         g[even] *= 2.0 ** (10 * ramp)
     elif kind == "matrix":
@@ -80,7 +83,7 @@ def boxes(n, few):
     return (61, 5, 1) if n == 8 or n >= 10 else ((61, 15, 1) if n >= 6 else (199, 3, 17))
 
 
-@pytest.mark.parametrize("kind", ["spike", "corner", "tiny", "jacobian", "matrix"])
+@pytest.mark.parametrize("kind", ["spike", "corner", "tiny", "flat", "jacobian", "matrix"])
 @pytest.mark.parametrize("few", [False, True])
 @pytest.mark.parametrize("n", [2, 5, 8, 10, 16])
 def test_operator(nek, oracle, n, few, kind):
