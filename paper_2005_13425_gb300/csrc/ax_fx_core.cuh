@@ -544,10 +544,15 @@ __device__ __forceinline__ void fx_final(const FxThread<N, G> &th, const int2 *X
 // tell, fx_grade), and so is every line along a direction whose factors are below
 // 2^-14 of the element's largest (sides 128 : 1; with t such a direction all
 // elements are listed, and at 2^-6 flat boxes of 16 layers to one ran 11 to 18 %
-// slower).  An element is graded if all three lines of some
-// point are small, leaving out lines of zeros along t (on a face of the box,
-// where a field vanishes) and points on the box's faces, which the CG heads
-// zero; or if all its entries are tiny (kMinExp), or its word says so.
+// slower).  A point is small if all three lines through it are, leaving out
+// lines of zeros along t (on a face of the box, where a field vanishes) and
+// points on the box's faces, which the CG heads zero.  An element is graded if
+// more than 1/64 of its points are small, or the lines through one are all below
+// 2^-16: the few points beside the corners of a box where a smooth field vanishes
+// (2^-8 at n = 8, 2^-14 at n = 16) are not worth another pass, whose latency is
+// that of the whole call on small boxes (64 elements at n = 8 12.3 us
+// instead of 8.2, of which 2 are the look at them).  And it is graded if all its entries are tiny (kMinExp), or its
+// word says so.
 // Why 8: on elements stretched by factors up to 100 and nine kinds of data
 // (emulated, n = 2 to 16) the largest error of a kept element is mostly below the
 // double-float operator's and at most 18 times as large (a single entry 2^7
@@ -644,28 +649,32 @@ __device__ __noinline__ void fx_redo_line(const float2 *in, float2 *out, int bas
     else line_plain<N>(in, out, base, stride, tr ? D->bwd : D->fwd);
 }
 
-// The lines through the points of a thread's column: are those along all three
-// directions small at one of the `points` (bits)?  X: the element's input in float
-// pairs, its largest entry in [1, 2).  weak: bits of directions whose lines all are.
+// The points of a thread's column through which the lines along all three directions
+// are small, of the `points` (bits): how many, or kFxFar if the lines through one are
+// all 2^-16 of the largest entry or less.  X: the element's input in float pairs,
+// its largest entry in [1, 2).  weak: bits of directions whose lines all are small.
+constexpr int kFxFar = 1 << 12;     // more than 1/64 of an element; 64 times all threads' sum fits an int
 template <int N, int G>
-__device__ __forceinline__ bool fx_small_lines(const FxThread<N, G> &th, const float2 *X, int weak, unsigned points) {
+__device__ __forceinline__ int fx_small_points(const FxThread<N, G> &th, const float2 *X, int weak, unsigned points) {
     constexpr int L = fx_layer(N);
-    auto small = [&](int dir, int at, int stride, bool zero_too) {
-        if ((weak >> dir) & 1) return true;
-        bool zero = true;
-#pragma unroll 1
-        for (int l = 0; l < N; l++) {
-            const float h = fabsf(X[at + l * stride].x);
-            if (h >= 2.f / (1 << fx_grade(N))) return false;
-            zero = zero && h == 0.f;
-        }
-        return zero_too || !zero;
+    constexpr float kSmall = 2.f / (1 << fx_grade(N));
+    auto top = [&](int dir, int at, int stride) {
+        float m = 0.f;
+#pragma unroll
+        for (int l = 0; l < N; l++) m = fmaxf(m, fabsf(X[at + l * stride].x));
+        return (weak >> dir) & 1 ? 0.f : m;
     };
-    if (!small(2, th.column(), L, false)) return false;
+    const float t = top(2, th.column(), L);
+    if (t >= kSmall || (t == 0.f && !((weak >> 2) & 1))) return 0;      // a line of zeros does not count
+    int count = 0;
 #pragma unroll 1
-    for (int k = 0; k < N; k++)
-        if (((points >> k) & 1u) && small(0, N * th.j + L * k, 1, true) && small(1, th.i + L * k, N, true)) return true;
-    return false;
+    for (int k = 0; k < N; k++) {
+        if (!((points >> k) & 1u)) continue;
+        const float m = fmaxf(t, fmaxf(top(0, N * th.j + L * k, 1), top(1, th.i + L * k, N)));
+        if (m < 0x1p-15f) return kFxFar;
+        count += m < kSmall;
+    }
+    return count;
 }
 
 // A CTA's list, when it has done its share: w = ax_e(v) in double-float arithmetic
@@ -681,7 +690,7 @@ __device__ __noinline__ void fx_redo_list(const FxData &fd, const FxList<fx_epc(
     constexpr int EPC = fx_epc(N, G);
     __shared__ int2 s_slot[EPC];       // the elements at work and their exponents
     __shared__ int s_next;
-    __shared__ unsigned s_graded;
+    __shared__ int s_small[EPC];       // their small points (fx_small_points)
     FxThread<N, G> th;
     th.init();
     const auto *D = (const typename DfConsts<N, EO>::type *)fd.dd;
@@ -708,8 +717,8 @@ __device__ __noinline__ void fx_redo_list(const FxData &fd, const FxList<fx_epc(
                 e = entry.x;
             }
             s_next = CHAIN ? e : -1;
-            s_graded = 0;
         }
+        if (threadIdx.x < EPC) s_small[threadIdx.x] = 0;
         __syncthreads();
         const int64_t e = s_slot[th.el].x;
         const int emax = s_slot[th.el].y;
@@ -733,11 +742,15 @@ __device__ __noinline__ void fx_redo_list(const FxData &fd, const FxList<fx_epc(
                 if (th.has(kk)) X[at + th.point(kk) * L] = dfa::split_scaled(x[kk], 1023 - emax);
         }
         __syncthreads();
-        if (on && ((word & kFxGraded) || emax <= fx::kMinExp ||
-                   fx_small_lines(th, X, word / kFxWeak, fx_inner_points(th, bf))))
-            atomicOr(&s_graded, 1u << th.el);
+        if (on) {
+            const int small = (word & kFxGraded) || emax <= fx::kMinExp
+                                  ? kFxFar
+                                  : fx_small_points(th, X, word / kFxWeak, fx_inner_points(th, bf));
+            if (small) atomicAdd(&s_small[th.el], small);
+        }
         __syncthreads();
-        on = on && ((s_graded >> th.el) & 1u);
+        // G = 3: a column's threads count its points three times
+        on = on && s_small[th.el] * 64 > G * N3;
         if (on) {
             if (G == 1 || th.d == 0) line(X, R, 0, false);
             if (G == 1 || th.d == 1) line(X, S, 1, false);
